@@ -9,7 +9,8 @@
 // read, so the compulsory HBM traffic is 8 links + 1 input + 1 output per
 // site.  The work is bandwidth-bound (0.36 flop/byte in FP64, 0.9 in
 // FP32/12), so there are no tensor cores here: the 3x3 complex mat-vecs run
-// on the FP32 / FP64 pipes in registers.
+// in registers, on the FP32 pipe or, for FP64, on the integer pipe
+// (fix64.cuh; 0.6 T FMA/s of FP64 would take 2.6 times the memory time).
 //
 // Reductions of FP64 data sum in FP64; those of FP32 / 16-bit data use the
 // compensated FP32 pairs of grid_sum_ff (the FP64 pipe is ~1/64 of FP32 here).
@@ -25,8 +26,14 @@
 
 namespace stg {
 
+// Limb links (fix64.cuh): two blocks per SM, 128 registers.  Measured at
+// 24^3x48, A with its dot, 18-real / 12-real: 145 / 208 us; three blocks (80
+// registers, 150-550 bytes spilled) 146 / 224 us; one block (200 registers)
+// 193 / 270 us.
+constexpr int min_blocks(int p, int r) { return p == P64 && (r & kFixLinks) ? 2 : 1; }
+
 template <int P, int R, int EPI>
-__global__ void __launch_bounds__(kBlock) k_dslash(const DslashArgs a)
+__global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const DslashArgs a)
 {
     typedef typename Real<P>::T T;
     pdl_wait();
@@ -141,7 +148,10 @@ stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &L
         STG_CUDA(cudaGetLastError());
         return STG_OK;
     }
-    if (prec == P64) {
+    if (prec == P64 && L.links->fix) {  // links as limbs: the integer form
+        if (recon == 18) launch_pr<P64, 18 | kFixLinks>(epi, a, grid, s, L.pdl);
+        else launch_pr<P64, 12 | kFixLinks>(epi, a, grid, s, L.pdl);
+    } else if (prec == P64) {
         if (recon == 18) launch_pr<P64, 18>(epi, a, grid, s, L.pdl);
         else launch_pr<P64, 12>(epi, a, grid, s, L.pdl);
     } else if (prec == P32) {

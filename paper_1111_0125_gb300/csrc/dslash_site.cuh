@@ -2,21 +2,22 @@
 // per-thread kernels (dslash.cu) and the multi-lattice group launch
 // (group.cu): the four forward links at the site, the four backward links at
 // the neighbours, the eight neighbour colour vectors, and for FX16 links the
-// scale 1/32767 applied once to the sum.
+// scale 1/32767 applied once to the sum.  FP64 links held as limbs (R has
+// kFixLinks) take the integer form of fix64.cuh.
 #pragma once
 
-#include "stg_internal.h"
+#include "fix64.cuh"
 
 namespace stg {
 
+// links and fields in floating point
 template <int P, int R>
-__device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site(const Geom &g, const char *const *lf,
-                                                                 const char *const *lb, int parity,
-                                                                 const void *in, int i)
+__device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site_fp(const Geom &g, const Site &s,
+                                                                    const char *const *lf,
+                                                                    const char *const *lb, const void *in, int i)
 {
     typedef typename Real<P>::T T;
     const int vh = g.Vh;
-    const Site s = site_of(g, i, parity);
     Vec3<T> acc;
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc.r[c] = acc.i[c] = T(0);
@@ -43,6 +44,25 @@ __device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site(const Geom &g, 
         }
     }
     return acc;
+}
+
+template <int P, int R>
+__device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site(const Geom &g, const char *const *lf,
+                                                                 const char *const *lb, int parity,
+                                                                 const void *in, int i)
+{
+    if constexpr (P == P64 && (R & kFixLinks) != 0) {
+        constexpr int RC = R & ~kFixLinks;
+        return fix_site<RC>(g, parity, i, [&](const Site &s, int i, int mu, bool back) {
+            int jf, jb;
+            neighbours(g, s, i, mu, jf, jb);
+            float sf = 1.f, sb = 1.f;
+            if (RC == 12) link_signs(g, s, mu, sf, sb);
+            return back ? FixHop{lb[mu], g.Vh, jb, in, g.Vh, jb, sb} : FixHop{lf[mu], g.Vh, i, in, g.Vh, jf, sf};
+        });
+    } else {
+        return dslash_site_fp<P, R>(g, site_of(g, i, parity), lf, lb, in, i);
+    }
 }
 
 }  // namespace stg

@@ -1,0 +1,293 @@
+// The FP64 Dslash half-pass at one output site on the integer pipe.
+//
+// This part of the chip multiplies FP64 at 2 per SM and clock but forms
+// 32 x 32 + 64-bit integer products (IMAD.WIDE) at 64: 0.60 against 19.1 T/s
+// measured.  The 288 FP64 FMAs of a site bound the FP64 half-pass at 2.6
+// times its memory time, so the mat-vecs run in fixed point instead, three
+// integer products for one FP64 product, 864 a site:
+//
+//   * A link entry is held as two limbs, u = h 2^-29 + l 2^-57, |h| <= 2^29,
+//     -2^27 <= l < 2^27 (k_fix_links, 8 bytes as the double it replaces).
+//     A link field takes this form only when every link is unitary to 1e-3
+//     (k_check_links); others keep doubles and the FP64 arithmetic.
+//   * A neighbour's colour vector is cut to 57 bits below 2^(E - 1022), E the
+//     largest FP64 exponent met so far at this site (all limbs of a component
+//     carry its sign).  When a later neighbour raises E the sums move right.
+//   * hh sums h h' and mm sums h l' + l h' in 64 bits; the l l' terms, below
+//     2^-60 of the largest component, are left out.  Unit rows give |hh| <
+//     8 sqrt(6) 2^58 < 2^63; |mm| < 48 2^56 + 20 2^57 < 2^63.
+//   * The total hh + (mm >> 28), up to 62 bits, becomes a double once: the
+//     rounding errors of 48 FMAs (2^-53 each) are replaced by input cuts of
+//     2^-57 of the largest neighbour component and one rounding.
+//
+// Measured (GB300, half-pass): 32^3x64 18-real 492 -> 199 us (6.58 TB/s, 0.97
+// of the measured copy rate), 24^3x48 18-real 168 -> 66 us, 12-real 326 -> 101
+// us (issue-bound: rebuilding row 2 is 576 more products a site), 8^4 21 -> 11
+// us.  Error of D D chi on Gaussian fields against 64-bit sums: 3.4e-16 ->
+// 1.8e-16 (norm), 3.1e-15 -> 1.5e-15 (largest component).
+//
+// Sites whose largest neighbour component is not finite, 2^1017 or more, or
+// below 2^-894 are recomputed in FP64 from the same data (zero vectors, as in
+// a point source's field, are skipped there).
+#pragma once
+
+#include "stg_internal.h"
+
+namespace stg {
+
+// R of the FP64 kernels: the reconstruction, with kFixLinks for limb links
+constexpr int kFixLinks = 256;
+
+struct FixLink {
+    int h[3][3][2], l[3][3][2];  // [row][column][re, im]
+};
+
+// v, in units of 2^-58, to limbs in units of 2^-29 and 2^-57
+__device__ __forceinline__ void fix_split(long long v, int &h, int &l)
+{
+    const long long x = (v + 1) >> 1;
+    h = (int)((x + (1 << 27)) >> 28);
+    l = (int)(x - ((long long)h << 28));
+}
+
+template <int N> struct FixDot {  // N products a b, to 2^-58
+    long long hh = 0, mm = 0;
+    __device__ __forceinline__ void add(int ah, int al, int bh, int bl)
+    {
+        hh += (long long)ah * bh;
+        mm += (long long)ah * bl;
+        mm += (long long)al * bh;
+    }
+};
+
+// row 2 = s conj(r0 x r1) from the limbs of rows 0 and 1
+__device__ __forceinline__ void fix_row2(FixLink &u, int s)
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int b = (a + 1) % 3, c = (a + 2) % 3;
+#define STG_L(r_, k_, z_) u.h[r_][k_][z_], u.l[r_][k_][z_]
+        FixDot<2> p, n;
+        p.add(STG_L(0, b, 0), STG_L(1, c, 0));
+        p.add(STG_L(0, c, 1), STG_L(1, b, 1));
+        n.add(STG_L(0, b, 1), STG_L(1, c, 1));
+        n.add(STG_L(0, c, 0), STG_L(1, b, 0));
+        long long re = (p.hh - n.hh) + ((p.mm - n.mm) >> 28);
+        FixDot<2> pi, ni;
+        pi.add(STG_L(0, b, 0), STG_L(1, c, 1));
+        pi.add(STG_L(0, b, 1), STG_L(1, c, 0));
+        ni.add(STG_L(0, c, 0), STG_L(1, b, 1));
+        ni.add(STG_L(0, c, 1), STG_L(1, b, 0));
+#undef STG_L
+        long long im = (ni.hh - pi.hh) + ((ni.mm - pi.mm) >> 28);
+        if (s < 0) {
+            re = -re;
+            im = -im;
+        }
+        fix_split(re, u.h[2][a][0], u.l[2][a][0]);
+        fix_split(im, u.h[2][a][1], u.l[2][a][1]);
+    }
+}
+
+template <int RC>
+__device__ __forceinline__ FixLink fix_link(const char *blk, int stride, int i, int s2)
+{
+    const uint4 *p = reinterpret_cast<const uint4 *>(blk) + i;
+    FixLink u;
+    constexpr int n = RC == 18 ? 9 : 6;
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+        const uint4 a = ld_stream(p + (size_t)k * stride);
+        u.h[k / 3][k % 3][0] = (int)a.x;
+        u.l[k / 3][k % 3][0] = (int)a.y;
+        u.h[k / 3][k % 3][1] = (int)a.z;
+        u.l[k / 3][k % 3][1] = (int)a.w;
+    }
+    if (RC == 12) fix_row2(u, s2);
+    return u;
+}
+
+struct FixAcc {
+    long long hh[6], mm[6];  // re, im of colour 0, 1, 2
+    int e;                   // FP64 exponent field of the scale
+};
+
+constexpr int kFixExpMin = 128, kFixExpMax = 2040;
+
+__device__ __forceinline__ void fix_init(FixAcc &a)
+{
+#pragma unroll
+    for (int k = 0; k < 6; ++k) a.hh[k] = a.mm[k] = 0;
+    a.e = kFixExpMin;
+}
+
+// limbs of v below 2^(e - 1022): v = (h 2^28 + l) 2^(e - 1079), both with the
+// sign of v (flipped with NEG); zero where v lies 57 or more bits below
+template <bool NEG>
+__device__ __forceinline__ void fix_cut(double v, int e, int &h, int &l)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned wh = __funnelshift_l(lo, hi, 11) | 0x80000000u, wl = lo << 11;
+    const unsigned long long w = ((unsigned long long)wh << 32) | wl;
+    const int n = e - (int)((hi >> 20) & 0x7ffu) + 7;  // a subnormal (field 0) is shifted out
+    unsigned long long x;
+    asm("shr.u64 %0, %1, %2;" : "=l"(x) : "l"(w), "r"(n));
+    const int m = NEG ? ~((int)hi >> 31) : (int)hi >> 31;
+    const int xl = (int)(unsigned)x & 0xfffffff;
+    const int xh = (int)__funnelshift_r((unsigned)x, (unsigned)(x >> 32), 28);
+    h = (xh ^ m) - m;
+    l = (xl ^ m) - m;
+}
+
+// acc += U v (forward) or acc -= U^dag v (ADJ); v in doubles
+template <bool ADJ>
+__device__ __forceinline__ void fix_hop(FixAcc &acc, const FixLink &u, const Vec3<double> &v)
+{
+    unsigned mx = 0u;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const unsigned a = (unsigned)__double2hiint(v.r[c]) & 0x7fffffffu;
+        const unsigned b = (unsigned)__double2hiint(v.i[c]) & 0x7fffffffu;
+        mx = max(mx, max(a, b));
+    }
+    const int e = (int)(mx >> 20);
+    if (e > acc.e) {
+        const int s = min(e - acc.e, 63);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            acc.hh[k] >>= s;
+            acc.mm[k] >>= s;
+        }
+        acc.e = e;
+    }
+    // ADJ: w = -v and its negated real parts; forward: v and its negated
+    // imaginary parts
+    int rh[3], rl[3], ih[3], il[3], nh[3], nl[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        fix_cut<ADJ>(v.r[c], acc.e, rh[c], rl[c]);
+        fix_cut<ADJ>(v.i[c], acc.e, ih[c], il[c]);
+        nh[c] = ADJ ? -rh[c] : -ih[c];
+        nl[c] = ADJ ? -rl[c] : -il[c];
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int p = ADJ ? b : a, q = ADJ ? a : b;
+            const int xh = u.h[p][q][0], xl = u.l[p][q][0], yh = u.h[p][q][1], yl = u.l[p][q][1];
+            long long &hr = acc.hh[2 * a], &mr = acc.mm[2 * a];
+            long long &hi = acc.hh[2 * a + 1], &mi = acc.mm[2 * a + 1];
+            hr += (long long)xh * rh[b];
+            mr += (long long)xh * rl[b];
+            mr += (long long)xl * rh[b];
+            hi += (long long)xh * ih[b];
+            mi += (long long)xh * il[b];
+            mi += (long long)xl * ih[b];
+            // forward: re -= y i, im += y r; ADJ: re += y w_i, im -= y w_r
+            const int ch = ADJ ? ih[b] : nh[b], cl = ADJ ? il[b] : nl[b];
+            const int dh = ADJ ? nh[b] : rh[b], dl = ADJ ? nl[b] : rl[b];
+            hr += (long long)yh * ch;
+            mr += (long long)yh * cl;
+            mr += (long long)yl * ch;
+            hi += (long long)yh * dh;
+            mi += (long long)yh * dl;
+            mi += (long long)yl * dh;
+        }
+}
+
+__device__ __forceinline__ bool fix_ok(const FixAcc &a) { return a.e < kFixExpMax && a.e > kFixExpMin; }
+
+// (hh + (mm >> 28)) 2^(e - 1080), rounded to nearest (half away from zero) by
+// integer operations: the conversion instruction runs on the FP64 pipe
+__device__ __forceinline__ double fix_double(long long hh, long long mm, int e)
+{
+    const long long v = hh + (mm >> 28);
+    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << (lz & 63);  // leading one at bit 63
+    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);  // a carry raises the exponent below
+    const unsigned long long r = m + ((unsigned long long)(unsigned)(e + 5 - lz) << 52);
+    const unsigned hi = (unsigned)(r >> 32) | ((unsigned)(v >> 32) & 0x80000000u);
+    return a ? __hiloint2double((int)hi, (int)(unsigned)r) : 0.0;
+}
+
+__device__ __forceinline__ Vec3<double> fix_value(const FixAcc &a)
+{
+    Vec3<double> v;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        v.r[c] = fix_double(a.hh[2 * c], a.mm[2 * c], a.e);
+        v.i[c] = fix_double(a.hh[2 * c + 1], a.mm[2 * c + 1], a.e);
+    }
+    return v;
+}
+
+// One hop's operands: the link record and the neighbour's vector, each by
+// base, plane stride and index, and the sign of a 12-real link's row 2.
+struct FixHop {
+    const char *link;
+    int lstride, li;
+    const void *f;
+    int fstride, fi;
+    float s;
+};
+
+// One hop in FP64 on the link's doubles (the recomputation): acc += U v, or
+// acc -= U^dag v for a backward hop.  Not inlined: it runs for exceptional
+// sites only, and inlined its registers made every site's path spill.
+template <int RC>
+__device__ __noinline__ void fix_hop_f64(const FixHop t, bool back, Vec3<double> *acc)
+{
+    const Vec3<double> v = FieldIO<P64>::load_nc(t.f, t.fstride, t.fi);
+    if (v.r[0] == 0.0 && v.i[0] == 0.0 && v.r[1] == 0.0 && v.i[1] == 0.0 && v.r[2] == 0.0 && v.i[2] == 0.0) return;
+    const uint4 *p = reinterpret_cast<const uint4 *>(t.link) + t.li;
+    Mat3<double> u;
+#pragma unroll
+    for (int k = 0; k < (RC == 18 ? 9 : 6); ++k) {
+        const uint4 a = ld_stream(p + (size_t)k * t.lstride);
+        set_entry(u, k, (double)(int)a.x * 0x1p-29 + (double)(int)a.y * 0x1p-57,
+                  (double)(int)a.z * 0x1p-29 + (double)(int)a.w * 0x1p-57);
+    }
+    if (RC == 12) reconstruct_row2(u, 1.0);
+    const double s = RC == 12 ? (double)t.s : 1.0;
+    Vec3<double> d = *acc;
+    if (back) adj_mul_sub(u, v, d, s);
+    else mul_add<RC == 12>(u, v, d, s);
+    *acc = d;
+}
+
+// D chi at site i; hop(s, i, mu, back) gives the eight hops' operands.
+template <int RC, class H>
+__device__ __forceinline__ Vec3<double> fix_site(const Geom &g, int parity, int i, const H &hop)
+{
+    const Site s = site_of(g, i, parity);
+    FixAcc acc;
+    fix_init(acc);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        {
+            const FixHop t = hop(s, i, mu, false);
+            const FixLink u = fix_link<RC>(t.link, t.lstride, t.li, t.s < 0.f ? -1 : 1);
+            fix_hop<false>(acc, u, FieldIO<P64>::load_nc(t.f, t.fstride, t.fi));
+        }
+        {
+            const FixHop t = hop(s, i, mu, true);
+            const FixLink u = fix_link<RC>(t.link, t.lstride, t.li, t.s < 0.f ? -1 : 1);
+            fix_hop<true>(acc, u, FieldIO<P64>::load_nc(t.f, t.fstride, t.fi));
+        }
+    }
+    if (fix_ok(acc)) return fix_value(acc);
+    // from the index alone (the empty asm): no neighbour address stays in a
+    // register for this branch
+    asm volatile("" : "+r"(i));
+    const Site z = site_of(g, i, parity);
+    Vec3<double> d;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d.r[c] = d.i[c] = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) fix_hop_f64<RC>(hop(z, i, k >> 1, k & 1), k & 1, &d);
+    return d;
+}
+
+}  // namespace stg

@@ -155,6 +155,70 @@ stg_status pack_links_flip(const Geom &g, const double2 *ucan, int prec, int rec
     return STG_OK;
 }
 
+// *bad = 1 unless every link U has |(U U^dag)_ij - delta_ij| <= 1e-3 (NaN
+// fails): the bound that the integer sums of fix64.cuh need
+__global__ void k_check_links(const double2 *__restrict__ ucan, long n, int *bad)
+{
+    const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    // FP32 is enough for the bound, and the FP64 pipe is slow
+    float2 u[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const double2 v = ucan[(size_t)k * 9 + q];
+        u[q] = make_float2((float)v.x, (float)v.y);
+    }
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j <= i; ++j) {
+            float re = i == j ? -1.f : 0.f, im = 0.f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float2 a = u[3 * i + c], b = u[3 * j + c];
+                re += a.x * b.x + a.y * b.y;
+                im += a.y * b.x - a.x * b.y;
+            }
+            ok = ok && fabsf(re) <= 1e-3f && fabsf(im) <= 1e-3f;
+        }
+    if (!ok) *bad = 1;
+}
+
+// doubles to limbs in place: u = h 2^-29 + l 2^-57, -2^27 <= l < 2^27
+__global__ void k_fix_links(long n, double2 *u)
+{
+    const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const double2 v = u[k];
+    const long long a = __double2ll_rn(v.x * 0x1p57), b = __double2ll_rn(v.y * 0x1p57);
+    int4 w;
+    w.x = (int)((a + (1 << 27)) >> 28);
+    w.y = (int)(a - ((long long)w.x << 28));
+    w.z = (int)((b + (1 << 27)) >> 28);
+    w.w = (int)(b - ((long long)w.z << 28));
+    reinterpret_cast<int4 *>(u)[k] = w;
+}
+
+stg_status links_check(const double2 *ucan, long n, int *bad, cudaStream_t s)
+{
+    k_check_links<<<(int)((n + 255) / 256), 256, 0, s>>>(ucan, n, bad);
+    STG_CUDA(cudaGetLastError());
+    return STG_OK;
+}
+
+stg_status links_fix(const Geom &g, LinkField *lf, cudaStream_t s)
+{
+    // every block holds Vh records in planes, all of them (re, im) pairs
+    const long n = (long)g.Vh * (link_bytes(P64, lf->recon) / 16);
+    for (int b = 0; b < 8; ++b)
+        k_fix_links<<<(int)((n + 255) / 256), 256, 0, s>>>(
+            n, reinterpret_cast<double2 *>(lf->base + (size_t)b * lf->blk_bytes));
+    STG_CUDA(cudaGetLastError());
+    lf->fix = true;
+    return STG_OK;
+}
+
 static stg_status pack_links(const Geom &g, const double2 *ucan, int prec, int recon,
                              LinkField *lf, cudaStream_t s)
 {
@@ -412,7 +476,8 @@ stg_status gauge_create(const int dims[4], const double *links_host, int sloppy,
     const size_t canon_bytes = (size_t)g->geom.Vh * 2 * 4 * 9 * sizeof(double2);
     double2 *ucan = nullptr;
     stg_status st = STG_OK;
-    e = cudaMalloc((void **)&ucan, canon_bytes);
+    // the canonical links and, behind them, the outcome of links_check
+    e = cudaMalloc((void **)&ucan, canon_bytes + 16);
     if (e != cudaSuccess) {
         delete g;
         set_error("stg_gauge_create: device staging allocation failed");
@@ -421,6 +486,13 @@ stg_status gauge_create(const int dims[4], const double *links_host, int sloppy,
     e = cudaMemcpyAsync(ucan, links_host, canon_bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) st = cuda_fail(e, "cudaMemcpyAsync(links)");
     const int recon_hi = (sloppy == P64) ? recon : 18;
+    int *bad_dev = reinterpret_cast<int *>(reinterpret_cast<char *>(ucan) + canon_bytes);
+    int bad = 1;
+    if (st == STG_OK && (e = cudaMemsetAsync(bad_dev, 0, sizeof(int), s)) != cudaSuccess)
+        st = cuda_fail(e, "cudaMemsetAsync");
+    if (st == STG_OK) st = links_check(ucan, (long)g->geom.Vh * 8, bad_dev, s);
+    if (st == STG_OK && (e = cudaMemcpyAsync(&bad, bad_dev, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+        st = cuda_fail(e, "cudaMemcpyAsync");
     if (st == STG_OK) st = pack_links(g->geom, ucan, P64, recon_hi, &g->hi, s);
     if (st == STG_OK && sloppy != P64) st = pack_links(g->geom, ucan, sloppy, recon, &g->lo, s);
     if (st == STG_OK && (sloppy == PX16 || sloppy == P16) && recon == 12 && want_tiled()) {
@@ -431,6 +503,11 @@ stg_status gauge_create(const int dims[4], const double *links_host, int sloppy,
         st = mtile_links(g->geom, &g->lo, s);
     e = cudaStreamSynchronize(s);
     if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
+    if (st == STG_OK && !bad) {
+        st = links_fix(g->geom, &g->hi, s);
+        e = cudaStreamSynchronize(s);
+        if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
+    }
     cudaFree(ucan);
     if (st != STG_OK) {
         if (g->hi.base) cudaFree(g->hi.base);

@@ -24,6 +24,7 @@ struct GroupItem {
     const void *in;
     void *out;
     int parity;
+    int fix;          // FP64 links as limbs (fix64.cuh)
     int first_block;  // the item's blocks are [first_block, next item's first_block)
 };
 
@@ -41,8 +42,11 @@ __global__ void __launch_bounds__(kBlock) k_dslash_group(const __grid_constant__
     const GroupItem &t = ga.it[p];
     const int i = ((int)blockIdx.x - t.first_block) * kBlock + (int)threadIdx.x;
     if (i >= t.g.Vh) return;
-    const auto acc = dslash_site<P, R>(t.g, t.lf, t.lb, t.parity, t.in, i);
-    FieldIO<P>::store(t.out, t.g.Vh, i, acc);
+    if (P == P64 && t.fix)
+        FieldIO<P>::store(t.out, t.g.Vh, i,
+                          dslash_site<P, P == P64 ? R | kFixLinks : R>(t.g, t.lf, t.lb, t.parity, t.in, i));
+    else
+        FieldIO<P>::store(t.out, t.g.Vh, i, dslash_site<P, R>(t.g, t.lf, t.lb, t.parity, t.in, i));
 }
 
 template <int P>
@@ -102,6 +106,7 @@ extern "C" stg_status stg_dslash_group(int n, const stg_gauge *const *g, const i
         t.in = in_dev[k];
         t.out = out_dev[k];
         t.parity = out_parity[k];
+        t.fix = lf->fix;
         t.first_block = (int)blocks;
         blocks += (gk->geom.Vh + kBlock - 1) / kBlock;
     }

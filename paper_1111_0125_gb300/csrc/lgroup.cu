@@ -43,6 +43,7 @@ struct LgEntry {
     size_t blk;
     char *y, *r, *d, *q, *t;
     int slot;             // index into the state array
+    int fix;              // FP64 links as limbs (fix64.cuh)
     int first_tile;       // this entry's items are [first_tile, first_tile + tiles)
     int tiles;
 };
@@ -132,7 +133,10 @@ __global__ void __launch_bounds__(kBlock, 2) k_lg_dslash(const LgArgs a)
         const int i = (w - e.first_tile) * kBlock + (int)threadIdx.x;
         T dot = T(0);
         if (i < vh) {
-            const Vec3<T> dv = dslash_site<P, R>(e.g, lf, lb, parity, EPI == EPI_GATE ? e.d : e.t, i);
+            const void *in = EPI == EPI_GATE ? e.d : e.t;
+            Vec3<T> dv;
+            if (P == P64 && e.fix) dv = dslash_site<P, P == P64 ? R | kFixLinks : R>(e.g, lf, lb, parity, in, i);
+            else dv = dslash_site<P, R>(e.g, lf, lb, parity, in, i);
             if (EPI == EPI_GATE) {
                 FieldIO<P>::store(e.t, vh, i, dv);
             } else {
@@ -419,6 +423,7 @@ static stg_status lg_push(stg_lgroup *b)
         const LinkField *lf = links_for(sl.g, b->pd);
         e.g = sl.g->geom;
         e.links = lf->base;
+        e.fix = lf->fix;
         e.blk = lf->blk_bytes;
         e.y = b->vec(k, stg_lgroup::Y);
         e.r = b->vec(k, stg_lgroup::R);

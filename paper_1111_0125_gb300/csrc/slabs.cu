@@ -177,6 +177,20 @@ __global__ void __launch_bounds__(kBlock) k_slab_collect(const CollectArgs a)
 // step 3: the Dslash of every slab (Eq. 5), the same arithmetic in the same
 // order as dslash_site, with the t-hops across a slab edge on the ghosts
 // ---------------------------------------------------------------------------
+// signs of a 12-real link's row 2 on a slab: eta_mu, and the antiperiodic
+// sign where the slab's edge is the lattice's
+__device__ __forceinline__ void slab_signs(const SlabDev *S, const Site &s, int mu, bool up, bool down, float &sf,
+                                           float &sb)
+{
+    int e = 0;
+    if (mu >= 1) e += s.x;
+    if (mu >= 2) e += s.y;
+    if (mu >= 3) e += s.z;
+    sf = sb = (e & 1) ? -1.f : 1.f;
+    if (up) sf *= S->top;
+    if (down) sb *= S->bot;
+}
+
 template <int P, int R>
 __device__ __forceinline__ Vec3<typename Real<P>::T> slab_site(const Geom &g, const SlabDev *S,
                                                                const char *const *lk, const char *const *gl,
@@ -184,45 +198,53 @@ __device__ __forceinline__ Vec3<typename Real<P>::T> slab_site(const Geom &g, co
 {
     typedef typename Real<P>::T T;
     const int vh = g.Vh, st = g.st, top = g.L[3] - 1;
-    const Site s = site_of(g, i, parity);
-    Vec3<T> acc;
+    if constexpr (P == P64 && (R & kFixLinks) != 0) {
+        constexpr int RC = R & ~kFixLinks;
+        return fix_site<RC>(g, parity, i, [&](const Site &s, int i, int mu, bool back) {
+            int jf, jb;
+            neighbours(g, s, i, mu, jf, jb);
+            const bool up = mu == 3 && s.t == top, down = mu == 3 && s.t == 0;
+            float sf = 1.f, sb = 1.f;
+            if (RC == 12) slab_signs(S, s, mu, up, down, sf, sb);
+            if (!back)
+                return up ? FixHop{lk[parity * 4 + mu], vh, i, S->recv[0], st, i - top * st, sf}
+                          : FixHop{lk[parity * 4 + mu], vh, i, in, vh, jf, sf};
+            return down ? FixHop{gl[parity], st, i, S->recv[1], st, i, sb}
+                        : FixHop{lk[(1 - parity) * 4 + mu], vh, jb, in, vh, jb, sb};
+        });
+    } else {
+        const Site s = site_of(g, i, parity);
+        Vec3<T> acc;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) acc.r[c] = acc.i[c] = T(0);
+        for (int c = 0; c < 3; ++c) acc.r[c] = acc.i[c] = T(0);
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        int jf, jb;
-        neighbours(g, s, i, mu, jf, jb);
-        const bool up = mu == 3 && s.t == top;  // x + t lies on the next slab
-        const bool down = mu == 3 && s.t == 0;  // x - t lies on the previous slab
-        float sf = 1.f, sb = 1.f;
-        if (R == 12) {
-            int e = 0;
-            if (mu >= 1) e += s.x;
-            if (mu >= 2) e += s.y;
-            if (mu >= 3) e += s.z;
-            sf = sb = (e & 1) ? -1.f : 1.f;
-            if (up) sf *= S->top;
-            if (down) sb *= S->bot;
+        for (int mu = 0; mu < 4; ++mu) {
+            int jf, jb;
+            neighbours(g, s, i, mu, jf, jb);
+            const bool up = mu == 3 && s.t == top;  // x + t lies on the next slab
+            const bool down = mu == 3 && s.t == 0;  // x - t lies on the previous slab
+            float sf = 1.f, sb = 1.f;
+            if (R == 12) slab_signs(S, s, mu, up, down, sf, sb);
+            const T s2f = (R == 12) ? T(sf * LinkPost<P>::row2) : T(1);
+            const T s2b = (R == 12) ? T(sb * LinkPost<P>::row2) : T(1);
+            const Mat3<T> uf = LinkIO<P, R>::load(lk[parity * 4 + mu], vh, i);
+            const Vec3<T> vf = up ? FieldIO<P>::load_nc(S->recv[0], st, i - top * st)
+                                  : FieldIO<P>::load_nc(in, vh, jf);
+            mul_add<R == 12>(uf, vf, acc, s2f);
+            const Mat3<T> ub = down ? LinkIO<P, R>::load(gl[parity], st, i)
+                                    : LinkIO<P, R>::load(lk[(1 - parity) * 4 + mu], vh, jb);
+            const Vec3<T> vb = down ? FieldIO<P>::load_nc(S->recv[1], st, i) : FieldIO<P>::load_nc(in, vh, jb);
+            adj_mul_sub(ub, vb, acc, s2b);
         }
-        const T s2f = (R == 12) ? T(sf * LinkPost<P>::row2) : T(1);
-        const T s2b = (R == 12) ? T(sb * LinkPost<P>::row2) : T(1);
-        const Mat3<T> uf = LinkIO<P, R>::load(lk[parity * 4 + mu], vh, i);
-        const Vec3<T> vf = up ? FieldIO<P>::load_nc(S->recv[0], st, i - top * st)
-                              : FieldIO<P>::load_nc(in, vh, jf);
-        mul_add<R == 12>(uf, vf, acc, s2f);
-        const Mat3<T> ub = down ? LinkIO<P, R>::load(gl[parity], st, i)
-                                : LinkIO<P, R>::load(lk[(1 - parity) * 4 + mu], vh, jb);
-        const Vec3<T> vb = down ? FieldIO<P>::load_nc(S->recv[1], st, i) : FieldIO<P>::load_nc(in, vh, jb);
-        adj_mul_sub(ub, vb, acc, s2b);
-    }
-    if (P == PX16) {
+        if (P == PX16) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            acc.r[c] *= T(LinkPost<PX16>::k);
-            acc.i[c] *= T(LinkPost<PX16>::k);
+            for (int c = 0; c < 3; ++c) {
+                acc.r[c] *= T(LinkPost<PX16>::k);
+                acc.i[c] *= T(LinkPost<PX16>::k);
+            }
         }
+        return acc;
     }
-    return acc;
 }
 
 // Epilogues as in dslash.cu: EPI_NONE / EPI_GATE store D in; EPI_A_DOT /
@@ -507,6 +529,7 @@ struct stg_slabs {
     int P = 0, prec = 0, recon = 18;
     Geom g;                          // local lattice (Lx, Ly, Lz, Lt / P)
     std::vector<LinkField> links;    // [P], in prec / recon
+    bool fix = false;                // FP64 links as limbs (fix64.cuh), all slabs alike
     std::vector<LinkField> links64;  // [P], FP64 / 18-real, when prec is not FP64
     char *ghost = nullptr;           // [P][2 output parities] ghost t-links
     size_t ghost_bytes = 0;
@@ -681,7 +704,15 @@ static stg_status sl_part(stg_slabs *h, int epi, SlabArgs a, int part, cudaStrea
     const dim3 grid((unsigned)nb, (unsigned)h->P);
     const bool r12 = a.recon == 12;
     switch (a.prec) {
-    case P64: if (r12) sl_launch_pr<P64, 12>(epi, grid, s, a); else sl_launch_pr<P64, 18>(epi, grid, s, a); break;
+    case P64:
+        if (h->fix) {
+            if (r12) sl_launch_pr<P64, 12 | kFixLinks>(epi, grid, s, a);
+            else sl_launch_pr<P64, 18 | kFixLinks>(epi, grid, s, a);
+        } else {
+            if (r12) sl_launch_pr<P64, 12>(epi, grid, s, a);
+            else sl_launch_pr<P64, 18>(epi, grid, s, a);
+        }
+        break;
     case P32: if (r12) sl_launch_pr<P32, 12>(epi, grid, s, a); else sl_launch_pr<P32, 18>(epi, grid, s, a); break;
     case P16: if (r12) sl_launch_pr<P16, 12>(epi, grid, s, a); else sl_launch_pr<P16, 18>(epi, grid, s, a); break;
     case PB16: if (r12) sl_launch_pr<PB16, 12>(epi, grid, s, a); else sl_launch_pr<PB16, 18>(epi, grid, s, a); break;
@@ -1109,12 +1140,24 @@ stg_status stg_slabs_create(const int dims[4], const double *links_host, int nsl
     // links of each slab, packed with the global sign rule (t_flip)
     const size_t canon_bytes = vh * 2 * 4 * 9 * sizeof(double2);
     double2 *ucan = nullptr;
-    stg_status st = sl_alloc((void **)&ucan, canon_bytes);
+    // the canonical links and, behind them, the outcome of links_check
+    stg_status st = sl_alloc((void **)&ucan, canon_bytes + 16);
+    int *bad_dev = reinterpret_cast<int *>(reinterpret_cast<char *>(ucan) + canon_bytes);
+    int bad = 1;
+    if (st == STG_OK) {
+        cudaError_t e = cudaMemsetAsync(bad_dev, 0, sizeof(int), s);
+        if (e != cudaSuccess) st = cuda_fail(e, "cudaMemsetAsync");
+    }
     for (int r = 0; r < P && st == STG_OK; ++r) {
         cudaError_t e = cudaMemcpyAsync(ucan, links_host + (size_t)r * (canon_bytes / sizeof(double)), canon_bytes,
                                         cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) st = cuda_fail(e, "cudaMemcpyAsync(links)");
         const int t_flip = r == P - 1 ? lts - 1 : -1;
+        if (st == STG_OK) st = links_check(ucan, (long)vh * 8, bad_dev, s);
+        if (st == STG_OK) {
+            e = cudaMemcpyAsync(&bad, bad_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
+            if (e != cudaSuccess) st = cuda_fail(e, "cudaMemcpyAsync");
+        }
         if (st == STG_OK) st = pack_links_flip(h->g, ucan, prec, recon, t_flip, &h->links[r], s);
         if (st == STG_OK && prec != STG_FP64) st = pack_links_flip(h->g, ucan, P64, 18, t_flip, &h->links64[r], s);
         if (st == STG_OK) {
@@ -1123,6 +1166,11 @@ stg_status stg_slabs_create(const int dims[4], const double *links_host, int nsl
         }
     }
     cudaFree(ucan);
+    if (st == STG_OK && !bad) {
+        for (int r = 0; r < P && st == STG_OK; ++r)
+            st = links_fix(h->g, prec != STG_FP64 ? &h->links64[r] : &h->links[r], s);
+        h->fix = true;
+    }
     if (st == STG_OK) st = sl_alloc((void **)&h->ghost, (size_t)P * 2 * h->ghost_bytes);
     if (st == STG_OK && prec != STG_FP64) st = sl_alloc((void **)&h->ghost64, (size_t)P * 2 * h->ghost64_bytes);
     if (st == STG_OK) st = sl_alloc((void **)&h->fields, (size_t)P * kSlabSlots * h->field_bytes);

@@ -55,6 +55,7 @@ struct LinkField {
     char *base = nullptr;   // 8 blocks: (parity, mu) -> base + (2 * 4 ... ) see blk()
     int prec = -1;
     int recon = 18;
+    bool fix = false;       // FP64: entries held as limbs (fix64.cuh) instead of doubles
     size_t blk_bytes = 0;   // bytes of one (parity, mu) block, 256-aligned
     char *tiled = nullptr;  // FX16 / 12-real only: tile-major copy (kFxTile)
     size_t tiled_parity_bytes = 0;
@@ -126,6 +127,12 @@ Geom make_geom(const int dims[4]);
 void cg_params_for(int sloppy, stg_cg_params *p);
 
 const LinkField *links_for(const stg_gauge *g, int prec);
+
+// FP64 links as limbs (gauge.cu): links_check raises *bad (device) where one
+// of n canonical links is not unitary; links_fix converts a packed FP64 field
+// in place
+stg_status links_check(const double2 *ucan, long n, int *bad, cudaStream_t s);
+stg_status links_fix(const Geom &g, LinkField *lf, cudaStream_t s);
 
 // Reduction scratch: partial sums (one double per block) and the state.
 struct Workspace {
