@@ -32,7 +32,7 @@ int grid_for(long n)
     return (int)(g < 1 ? 1 : g);
 }
 
-static int num_sms()
+int num_sms()
 {
     static const int n = [] {
         int dev = 0, m = 0;

@@ -138,13 +138,7 @@ stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &L
         set_error("dslash: link precision does not match the field precision");
         return STG_ERR_UNSUPPORTED;
     }
-    if (prec == PX16) {  // two sites per thread on packed FP32x2 (dslash_fx16.cu)
-        launch_dslash_fx2(recon, epi, a, s, L.pdl);
-        STG_CUDA(cudaGetLastError());
-        return STG_OK;
-    }
-    if (prec == P16 && recon == 12 && a.lt) {  // the same staged kernel, binary16 records
-        launch_dslash_f16_staged(epi, a, s, L.pdl);
+    if ((prec == PX16 || prec == P16) && launch_dslash_16(prec, recon, epi, a, s, L.pdl)) {
         STG_CUDA(cudaGetLastError());
         return STG_OK;
     }
@@ -161,6 +155,9 @@ stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &L
         if (prec == PB16) {
             if (recon == 18) launch_pr<PB16, 18>(epi, a, grid, s, L.pdl);
             else launch_pr<PB16, 12>(epi, a, grid, s, L.pdl);
+        } else if (prec == PX16) {
+            if (recon == 18) launch_pr<PX16, 18>(epi, a, grid, s, L.pdl);
+            else launch_pr<PX16, 12>(epi, a, grid, s, L.pdl);
         } else if (recon == 18) {
             launch_pr<P16, 18>(epi, a, grid, s, L.pdl);
         } else {

@@ -10,8 +10,9 @@
 // __fadd2_rn, __fmul2_rn) for both sites.  Loads of A and B are separate and
 // stay coalesced across the warp.
 //
-// The packed arithmetic (decode, 12-real reconstruction, mat-vecs, FX16
-// encode) is in fx16_pair.cuh.
+// This serves 12-real links; uncompressed ones run one site per thread
+// (dslash.cu).  The packed arithmetic (decode, 12-real reconstruction,
+// mat-vecs, FX16 encode) is in fx16_pair.cuh.
 #include "fx16_pair.cuh"
 
 #ifndef STG_FX2_MINBLOCKS
@@ -100,7 +101,7 @@ __device__ __forceinline__ f2 finish_pair(const DslashArgs &a, int iA, int iB, b
     return epilogue2<EPI, P>(a, iA, iB, okA, okB, dr, di, m2, wA, wB);
 }
 
-template <int R, int EPI>
+template <int EPI>
 __global__ void __launch_bounds__(kBlock, STG_FX2_MINBLOCKS) k_dslash_fx2(const DslashArgs a)
 {
     pdl_wait();
@@ -132,23 +133,20 @@ __global__ void __launch_bounds__(kBlock, STG_FX2_MINBLOCKS) k_dslash_fx2(const 
             int jfA, jbA, jfB, jbB;
             neighbours(a.g, sA, jA, mu, jfA, jbA);
             neighbours(a.g, sB, jB, mu, jfB, jbB);
-            f2 s2f = make_float2(1.f, 1.f), s2b = make_float2(1.f, 1.f);
-            if (R == 12) {
-                float sfA, sbA, sfB, sbB;
-                link_signs(a.g, sA, mu, sfA, sbA);
-                link_signs(a.g, sB, mu, sfB, sbB);
-                const float k = LinkPost<PX16>::row2;
-                s2f = make_float2(sfA * k, sfB * k);
-                s2b = make_float2(sbA * k, sbB * k);
-            }
+            float sfA, sbA, sfB, sbB;
+            link_signs(a.g, sA, mu, sfA, sbA);
+            link_signs(a.g, sB, mu, sfB, sbB);
+            const float k = LinkPost<PX16>::row2;
+            const f2 s2f = make_float2(sfA * k, sfB * k);
+            const f2 s2b = make_float2(sbA * k, sbB * k);
             Mat3x2 u;
             Vec3x2 v;
-            load_link2<R>(a.lf[mu], vh, jA, jB, u);
+            load_link2(a.lf[mu], vh, jA, jB, u);
             load_field2(a.in, jfA, jfB, v);
-            fwd2<R>(u, v, s2f, A);
-            load_link2<R>(a.lb[mu], vh, jbA, jbB, u);
+            fwd2<12>(u, v, s2f, A);
+            load_link2(a.lb[mu], vh, jbA, jbB, u);
             load_field2(a.in, jbA, jbB, v);
-            bwd2<R>(u, v, s2b, A);
+            bwd2<12>(u, v, s2b, A);
         }
         const float m2 = (EPI == EPI_A_CG) ? float(a.state->m2) : float(a.m2);
         f2 dA_B;
@@ -441,16 +439,16 @@ static void launch_staged(const DslashArgs &a, cudaStream_t s, bool pdl)
     launch_k(k_dslash_fx2_staged<P, EPI>, grid, kFxCons, kFxSmem, s, pdl, a);
 }
 
-template <int R>
-static void launch_r(int epi, const DslashArgs &a, int grid, cudaStream_t s, bool pdl)
+static void launch_pair(int epi, const DslashArgs &a, cudaStream_t s, bool pdl)
 {
+    const int grid = (a.g.Vh + 2 * kBlock - 1) / (2 * kBlock);
     switch (epi) {
-    case EPI_NONE: launch_k(k_dslash_fx2<R, EPI_NONE>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A: launch_k(k_dslash_fx2<R, EPI_A>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A_DOT: launch_k(k_dslash_fx2<R, EPI_A_DOT>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A_CG: launch_k(k_dslash_fx2<R, EPI_A_CG>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_RES: launch_k(k_dslash_fx2<R, EPI_RES>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_GATE: launch_k(k_dslash_fx2<R, EPI_GATE>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_NONE: launch_k(k_dslash_fx2< EPI_NONE>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_A: launch_k(k_dslash_fx2< EPI_A>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_A_DOT: launch_k(k_dslash_fx2< EPI_A_DOT>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_A_CG: launch_k(k_dslash_fx2< EPI_A_CG>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_RES: launch_k(k_dslash_fx2< EPI_RES>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_GATE: launch_k(k_dslash_fx2< EPI_GATE>, grid, kBlock, 0, s, pdl, a); break;
     }
 }
 
@@ -467,22 +465,42 @@ static void launch_staged_p(int epi, const DslashArgs &a, cudaStream_t s, bool p
     }
 }
 
-// IEEE FP16 / 12-real links in the tile-major copy: the staged kernel with
-// binary16 decode and encode
-void launch_dslash_f16_staged(int epi, const DslashArgs &a, cudaStream_t s, bool pdl)
+// Which kernel runs FP16 and FX16 half-passes.  The staged kernel gives each
+// SM whole tiles of 1024 sites, a round of them per 5.3 us, and so wastes the
+// last round: the kernels without staging take 0.039 us per 1024 sites at any
+// size, the staged one 5.3 us per started round of one tile per SM.  It wins
+// where at least 0.9 of its rounds is filled, and from five rounds on (before
+// that the first fill's latency shows).  Measured (half-pass / A with its dot,
+// FP16/12, us, staged against one site per thread): Vh 20736: 6.9 / 15.8
+// against 2.7 / 7.5; 65536: 7.2 / 18.5 against 4.4 / 10.7; 331776: 18.5 / 39.7
+// against 14.5 / 33.8; 786432 (5.05 rounds): 32.0 / 67.3 against 30.1 / 67.8;
+// 1048576 (6.74): 37.3 / 79.2 against 39.2 / 87.7.  The capped and the
+// withheld-fill grids of the tests always run staged.
+static bool staged_pays(const DslashArgs &a)
 {
-    launch_staged_p<P16>(epi, a, s, pdl);
+    if (!a.lt) return false;
+    if (a.grid_cap > 0 || a.drop_fill) return true;
+    const int slots = num_sms() * kFxCtasPerSM;
+    const int ntiles = (a.g.Vh + kFxTile - 1) / kFxTile;
+    const int rounds = (ntiles + slots - 1) / slots;
+    return rounds > 5 && 10L * ntiles >= 9L * slots * rounds;
 }
 
-void launch_dslash_fx2(int recon, int epi, const DslashArgs &a, cudaStream_t s, bool pdl)
+// Without staging, FX16/12 takes the packed kernel; the others one site per
+// thread: FX16/18 half-pass 2.5-47.1 us against the packed kernel's 3.8-48.5
+// (Vh 2048-1048576), FP16/12 within 3% of it from Vh 200000 and up to a third
+// faster below.
+bool launch_dslash_16(int prec, int recon, int epi, const DslashArgs &a, cudaStream_t s, bool pdl)
 {
-    if (recon == 12 && a.lt) {
-        launch_staged_p<PX16>(epi, a, s, pdl);
-        return;
+    if (recon != 12) return false;
+    if (staged_pays(a)) {
+        if (prec == P16) launch_staged_p<P16>(epi, a, s, pdl);
+        else launch_staged_p<PX16>(epi, a, s, pdl);
+        return true;
     }
-    const int grid = (a.g.Vh + 2 * kBlock - 1) / (2 * kBlock);
-    if (recon == 18) launch_r<18>(epi, a, grid, s, pdl);
-    else launch_r<12>(epi, a, grid, s, pdl);
+    if (prec == P16) return false;
+    launch_pair(epi, a, s, pdl);
+    return true;
 }
 
 }  // namespace stg

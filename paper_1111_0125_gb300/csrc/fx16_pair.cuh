@@ -98,28 +98,13 @@ __device__ __forceinline__ void decode12(const uint4 &a, const uint4 &b, const u
     }
 }
 
-// link of site A (index sa) and site B (index sb) of one (parity, mu) block
-template <int R>
+// 12-real FX16 link of site A (index sa) and site B (index sb) of one
+// (parity, mu) block
 __device__ __forceinline__ void load_link2(const char *blk, int vh, int sa, int sb, Mat3x2 &u)
 {
     const uint4 *p = reinterpret_cast<const uint4 *>(blk);
-    const uint4 a = ld_stream(p + sa), b = ld_stream(p + sb);
-    if (R == 18) {
-        set2(u, 0, a.x, b.x);
-        set2(u, 1, a.y, b.y);
-        set2(u, 2, a.z, b.z);
-        set2(u, 3, a.w, b.w);
-        const uint4 c = ld_stream(p + (size_t)vh + sa), d = ld_stream(p + (size_t)vh + sb);
-        set2(u, 4, c.x, d.x);
-        set2(u, 5, c.y, d.y);
-        set2(u, 6, c.z, d.z);
-        set2(u, 7, c.w, d.w);
-        const unsigned *q = reinterpret_cast<const unsigned *>(p + (size_t)2 * vh);
-        set2(u, 8, ld_stream(q + sa), ld_stream(q + sb));
-    } else {
-        const uint2 *q = reinterpret_cast<const uint2 *>(p + (size_t)vh);
-        decode12(a, b, ld_stream(q + sa), ld_stream(q + sb), u);
-    }
+    const uint2 *q = reinterpret_cast<const uint2 *>(p + (size_t)vh);
+    decode12(ld_stream(p + sa), ld_stream(p + sb), ld_stream(q + sa), ld_stream(q + sb), u);
 }
 
 // value = (u - 1.5 * 2^23 - 32768) s: the offset removed by one add and the

@@ -354,9 +354,9 @@ static bool want_mtiled()
     return !(v && v[0] == '0');
 }
 
-// The staged FX16 / FP16 12-real Dslash is the default; STG_FX16_TILED=0 at
-// gauge creation keeps the register-fed (FX16) or one-site (FP16) kernel (no
-// tile-major copy).
+// The tile-major copy lets large FX16 / FP16 12-real lattices run the staged
+// Dslash (staged_pays, dslash_fx16.cu); STG_FX16_TILED=0 at gauge creation
+// leaves it out (the register-fed FX16 or one-site FP16 kernel at any size).
 static bool want_tiled()
 {
     const char *v = getenv("STG_FX16_TILED");

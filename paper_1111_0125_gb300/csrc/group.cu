@@ -7,7 +7,8 @@
 // launch of their own; grouped, they fill it in one launch.  The per-site
 // arithmetic is dslash_site, so an item's output is bitwise the one of
 // stg_dslash wherever that runs the one-site-per-thread kernel (FX16 /
-// 12-real runs the packed staged kernel instead: equal to rounding).
+// 12-real and large FP16 / 12-real lattices run packed kernels instead: equal
+// to rounding).
 //
 // The paper applies the operator to one lattice at a time; this is a
 // serving-layer form of the same operation.

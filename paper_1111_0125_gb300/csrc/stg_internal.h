@@ -202,12 +202,12 @@ struct DslashArgs {
     unsigned *counter;
 };
 
-// FX16 Dslash, two sites per thread on packed FP32x2 arithmetic
-void launch_dslash_fx2(int recon, int epi, const DslashArgs &a, cudaStream_t s, bool pdl);
-// IEEE FP16 / 12-real with the tile-major links: the same staged kernel
-void launch_dslash_f16_staged(int epi, const DslashArgs &a, cudaStream_t s, bool pdl);
+// FP16 / FX16 Dslash on packed FP32x2 arithmetic (dslash_fx16.cu); false
+// where the one-site kernel of dslash.cu is the faster one
+bool launch_dslash_16(int prec, int recon, int epi, const DslashArgs &a, cudaStream_t s, bool pdl);
 
 int grid_for(long n);
+int num_sms();  // of the device current at the first call
 
 // vector-kernel helpers with explicit operands (cg.cu)
 int vec_grid(long n, int pd);
