@@ -53,11 +53,14 @@ constexpr int kVecBlocksPerSM = 2;
 // doubled registers would spill at 4)
 __host__ __device__ constexpr int vec_unroll(int pr) { return pr == P64 ? 2 : 4; }
 
-static int grid_vec(long n, int pr)
+// blocks per system of nsys systems
+static int grid_vec(long n, int nsys)
 {
-    const long u = vec_unroll(pr);
-    long g = (n + (long)kBlock * u - 1) / ((long)kBlock * u);
-    long cap = (long)num_sms() * kVecBlocksPerSM;
+    // one site per thread while the blocks last: the kernels are latency-bound
+    // there (16^3x32: 256 blocks, not 64 of four sites a thread)
+    long g = (n + kBlock - 1) / kBlock;
+    long cap = (long)num_sms() * kVecBlocksPerSM / nsys;
+    if (cap > kRrPartials) cap = kRrPartials;
     if (g > cap) g = cap;
     return (int)(g < 1 ? 1 : g);
 }
@@ -65,21 +68,22 @@ static int grid_vec(long n, int pr)
 // ---------------------------------------------------------------------------
 // vector kernels (grid-stride, FP64 reductions)
 // ---------------------------------------------------------------------------
+// dq: block partials of d^dag q; rr: this kernel's partials of |r|^2, one per
+// block (FP32 pairs unless the vectors are FP64)
 template <int PD, int PR>
 __device__ __forceinline__ void cg_update_body(int vh, void *y, void *r, const void *d, const void *q,
-                                               CGState *st, double *partials)
+                                               CGState *st, const double *dq, double *rr)
 {
-    if (st->flag != FLAG_RUN) return;
+    // one answer per block: block 0 may raise the flag below while others start
+    if (!__syncthreads_and(*(volatile const int *)&st->flag == FLAG_RUN)) return;
     typedef typename Real<PR>::T T;
     typedef typename Real<PD>::T TD;
     constexpr int kVecUnroll = vec_unroll(PR);
-    const T alpha = T(st->alpha);
-    double rr64 = 0.0;
-    FF rr = {0.f, 0.f};
     const int stride = gridDim.x * kBlock;
-    for (int base = blockIdx.x * kBlock + threadIdx.x; base < vh; base += kVecUnroll * stride) {
-        Vec3<TD> dv[kVecUnroll], qv[kVecUnroll];
-        Vec3<T> yv[kVecUnroll], rv[kVecUnroll];
+    int base = blockIdx.x * kBlock + threadIdx.x;
+    Vec3<TD> dv[kVecUnroll], qv[kVecUnroll];
+    Vec3<T> yv[kVecUnroll], rv[kVecUnroll];
+    const auto fetch = [&] {
 #pragma unroll
         for (int k = 0; k < kVecUnroll; ++k) {
             const int i = base + k * stride;
@@ -90,6 +94,27 @@ __device__ __forceinline__ void cg_update_body(int vh, void *y, void *r, const v
                 rv[k] = FieldIO<PR>::load(r, vh, i);
             }
         }
+    };
+    fetch();
+    __shared__ T sm_alpha;
+    __shared__ int sm_ok;
+    const double pAp = sum_partials<kBlock, PD != P64>(dq, st->n_part);
+    if (threadIdx.x == 0) {
+        double a;
+        sm_ok = cg_alpha(st->c_delta, pAp, st->m2, a);
+        sm_alpha = T(a);
+        if (blockIdx.x == 0) {
+            st->pAp = pAp;
+            if (sm_ok) st->alpha = a;
+            else st->flag = FLAG_BREAKDOWN;
+        }
+    }
+    __syncthreads();
+    if (!sm_ok) return;
+    const T alpha = sm_alpha;
+    double s64 = 0.0;
+    FF s = {0.f, 0.f};
+    while (base < vh) {
 #pragma unroll
         for (int k = 0; k < kVecUnroll; ++k) {
             const int i = base + k * stride;
@@ -106,69 +131,60 @@ __device__ __forceinline__ void cg_update_body(int vh, void *y, void *r, const v
                 T n = T(0);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) n += rs.r[c] * rs.r[c] + rs.i[c] * rs.i[c];
-                if constexpr (PR == P64) {
-                    rr64 += n;
-                } else {
-                    FF t;
-                    t.hi = float(n);
-                    t.lo = 0.f;
-                    rr = ff_add(rr, t);
-                }
+                if constexpr (PR == P64) s64 += n;
+                else s = ff_add(s, FF{float(n), 0.f});
             }
         }
+        base += kVecUnroll * stride;
+        if (base < vh) fetch();
     }
-    double total;
-    bool last;
-    if constexpr (PR == P64) last = grid_sum<kBlock>(rr64, partials, &st->counter, total);
-    else last = grid_sum_ff<kBlock>(rr, reinterpret_cast<float2 *>(partials), &st->counter, total);
-    if (last) {
-        const double old = st->delta_new;
-        st->delta_old = old;
-        st->delta_new = total;
-        st->beta = total / old;
-        st->iter += 1;
-        if (!isfinite(total)) st->flag = FLAG_BREAKDOWN;
-        else if (total <= st->stop_r2) st->flag = FLAG_CONVERGED;
-        else if (st->trig2 > 0.0 && total < st->trig2 * st->rmax2) st->flag = FLAG_UPDATE;
-        else if (st->iter >= st->iter_limit) st->flag = FLAG_MAXITER;
-        if (st->track_max && total > st->rmax2) st->rmax2 = total;
+    if constexpr (PR == P64) {
+        __shared__ double sm[kBlock];
+        const double t = block_sum_smem<kBlock>(s64, sm);
+        if (threadIdx.x == 0) rr[blockIdx.x] = t;
+    } else {
+        __shared__ float2 smf[32];
+        const FF t = block_sum_ff<kBlock>(s, smf);
+        if (threadIdx.x == 0) reinterpret_cast<float2 *>(rr)[blockIdx.x] = make_float2(t.hi, t.lo);
     }
 }
 
 template <int PD, int PR>
 __global__ void __launch_bounds__(kBlock, kVecBlocksPerSM)
-k_cg_update(int vh, void *y, void *r, const void *d, const void *q, CGState *st, double *partials)
+k_cg_update(int vh, void *y, void *r, const void *d, const void *q, CGState *st, const double *dq, double *rr)
 {
     pdl_wait();
     pdl_trigger();
-    cg_update_body<PD, PR>(vh, y, r, d, q, st, partials);
+    cg_update_body<PD, PR>(vh, y, r, d, q, st, dq, rr);
 }
 
-// several systems: blockIdx.y is the slot in the active list
+// several systems: blockIdx.y is the slot in the active list; the partials of
+// system k start at k times their number per system
 template <int PD, int PR>
 __global__ void __launch_bounds__(kBlock, kVecBlocksPerSM)
 k_cg_update_m(int vh, char *y, char *r, const char *d, const char *q, size_t sr, size_t sd,
-              CGState *states, double *partials, size_t pstride, const int *active,
-              const int *nactive)
+              CGState *states, const double *dq, double *rr, const int *active, const int *nactive)
 {
     if ((int)blockIdx.y >= *nactive) return;
     const int k = active[blockIdx.y];
     cg_update_body<PD, PR>(vh, y + k * sr, r + k * sr, d + k * sd, q + k * sd, states + k,
-                           partials + k * pstride);
+                           dq + (size_t)k * states[k].n_part, rr + (size_t)k * gridDim.x);
 }
 
+// beta = |r|^2 / delta and the stop tests from the update's partials (the
+// launch has the update's grid), then d = r + beta d
 template <int PD, int PR>
-__device__ __forceinline__ void xpay_body(int vh, const void *r, void *d, const CGState *st)
+__device__ __forceinline__ void xpay_body(int vh, const void *r, void *d, CGState *st, const double *rr)
 {
-    if (st->flag != FLAG_RUN) return;
+    if (!__syncthreads_and(*(volatile const int *)&st->flag == FLAG_RUN)) return;  // as in cg_update_body
     typedef typename Real<PR>::T T;
     typedef typename Real<PD>::T TD;
     constexpr int kVecUnroll = vec_unroll(PR);
-    const T beta = T(st->beta);
     const int stride = gridDim.x * kBlock;
-    for (int base = blockIdx.x * kBlock + threadIdx.x; base < vh; base += kVecUnroll * stride) {
-        Vec3<T> rv[kVecUnroll];
-        Vec3<TD> dv[kVecUnroll];
+    int base = blockIdx.x * kBlock + threadIdx.x;
+    Vec3<T> rv[kVecUnroll];
+    Vec3<TD> dv[kVecUnroll];
+    const auto fetch = [&] {
 #pragma unroll
         for (int k = 0; k < kVecUnroll; ++k) {
             const int i = base + k * stride;
@@ -177,6 +193,35 @@ __device__ __forceinline__ void xpay_body(int vh, const void *r, void *d, const 
                 dv[k] = FieldIO<PD>::load(d, vh, i);
             }
         }
+    };
+    fetch();
+    __shared__ T sm_beta;
+    __shared__ int sm_run;
+    const double total = sum_partials<kBlock, PR != P64>(rr, gridDim.x);
+    if (threadIdx.x == 0) {
+        const double old = st->c_delta;
+        const double beta = total / old;
+        const long long iter = st->c_iter + 1;
+        int flag = FLAG_RUN;
+        if (!isfinite(total)) flag = FLAG_BREAKDOWN;
+        else if (total <= st->stop_r2) flag = FLAG_CONVERGED;
+        else if (st->trig2 > 0.0 && total < st->trig2 * st->c_rmax2) flag = FLAG_UPDATE;
+        else if (iter >= st->iter_limit) flag = FLAG_MAXITER;
+        sm_beta = T(beta);
+        sm_run = flag == FLAG_RUN;
+        if (blockIdx.x == 0) {
+            st->delta_old = old;
+            st->delta_new = total;
+            st->beta = beta;
+            st->iter = iter;
+            if (st->track_max && total > st->c_rmax2) st->rmax2 = total;
+            if (flag != FLAG_RUN) st->flag = flag;
+        }
+    }
+    __syncthreads();
+    if (!sm_run) return;
+    const T beta = sm_beta;
+    while (base < vh) {
 #pragma unroll
         for (int k = 0; k < kVecUnroll; ++k) {
             const int i = base + k * stride;
@@ -190,26 +235,28 @@ __device__ __forceinline__ void xpay_body(int vh, const void *r, void *d, const 
                 FieldIO<PD>::store(d, vh, i, o);
             }
         }
+        base += kVecUnroll * stride;
+        if (base < vh) fetch();
     }
 }
 
 template <int PD, int PR>
 __global__ void __launch_bounds__(kBlock, kVecBlocksPerSM)
-k_xpay(int vh, const void *r, void *d, const CGState *st)
+k_xpay(int vh, const void *r, void *d, CGState *st, const double *rr)
 {
     pdl_wait();
     pdl_trigger();
-    xpay_body<PD, PR>(vh, r, d, st);
+    xpay_body<PD, PR>(vh, r, d, st, rr);
 }
 
 template <int PD, int PR>
 __global__ void __launch_bounds__(kBlock, kVecBlocksPerSM)
-k_xpay_m(int vh, const char *r, char *d, size_t sr, size_t sd, const CGState *states,
+k_xpay_m(int vh, const char *r, char *d, size_t sr, size_t sd, CGState *states, const double *rr,
          const int *active, const int *nactive)
 {
     if ((int)blockIdx.y >= *nactive) return;
     const int k = active[blockIdx.y];
-    xpay_body<PD, PR>(vh, r + k * sr, d + k * sd, states + k);
+    xpay_body<PD, PR>(vh, r + k * sr, d + k * sd, states + k, rr + (size_t)k * gridDim.x);
 }
 
 // x64 += y  (reliable update, Sec. 3.2: x_{k+1} = x_k + y_n in FP64)
@@ -366,10 +413,11 @@ static stg_status iteration(stg_gauge *gg, Workspace *ws, int pd, cudaStream_t s
     L.w = ws->d;
     STG_TRY(launch_dslash(g, pd, EPI_A_CG, L, s));
     if (ev) STG_CUDA(cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal));
-    const int grid = grid_vec(g.Vh, pr_of(pd));
-    STG_DISPATCH_PD_EX(pd, k_cg_update, pdl, g.Vh, ws->y, ws->r, ws->d, ws->q, ws->state, ws->partials);
+    const int grid = grid_vec(g.Vh, 1);
+    STG_DISPATCH_PD_EX(pd, k_cg_update, pdl, g.Vh, ws->y, ws->r, ws->d, ws->q, ws->state, ws->partials,
+                       ws->rr);
     if (ev) STG_CUDA(cudaEventRecordWithFlags(ev[3], s, cudaEventRecordExternal));
-    STG_DISPATCH_PD_EX(pd, k_xpay, pdl, g.Vh, ws->r, ws->d, ws->state);
+    STG_DISPATCH_PD_EX(pd, k_xpay, pdl, g.Vh, ws->r, ws->d, ws->state, ws->rr);
     if (ev) STG_CUDA(cudaEventRecordWithFlags(ev[4], s, cudaEventRecordExternal));
     STG_CUDA(cudaGetLastError());
     return STG_OK;
@@ -384,37 +432,21 @@ static stg_status cuda_check_launch()
 // ---------------------------------------------------------------------------
 // launch helpers with explicit operands (used by the multi-system solver)
 // ---------------------------------------------------------------------------
-int vec_grid(long n, int pd) { return grid_vec(n, pr_of(pd)); }
-
 stg_status launch_update_m(int pd, int vh, char *y, char *r, const char *d, const char *q, size_t sr,
-                           size_t sd, CGState *states, double *partials, size_t pstride,
-                           const int *active, const int *nactive, int nslots, cudaStream_t s)
+                           size_t sd, CGState *states, const double *dq, double *rr, const int *active,
+                           const int *nactive, int nslots, cudaStream_t s)
 {
-    const dim3 grid(grid_vec(vh, pr_of(pd)), nslots);
-    if (pd == P64)
-        k_cg_update_m<P64, P64><<<grid, kBlock, 0, s>>>(vh, y, r, d, q, sr, sd, states, partials, pstride, active, nactive);
-    else if (pd == P32)
-        k_cg_update_m<P32, P32><<<grid, kBlock, 0, s>>>(vh, y, r, d, q, sr, sd, states, partials, pstride, active, nactive);
-    else if (pd == P16)
-        k_cg_update_m<P16, P32><<<grid, kBlock, 0, s>>>(vh, y, r, d, q, sr, sd, states, partials, pstride, active, nactive);
-    else if (pd == PB16)
-        k_cg_update_m<PB16, P32><<<grid, kBlock, 0, s>>>(vh, y, r, d, q, sr, sd, states, partials, pstride, active, nactive);
-    else
-        k_cg_update_m<PX16, P32><<<grid, kBlock, 0, s>>>(vh, y, r, d, q, sr, sd, states, partials, pstride, active, nactive);
+    const dim3 grid(grid_vec(vh, nslots), nslots);
+    STG_DISPATCH_PD(pd, k_cg_update_m, vh, y, r, d, q, sr, sd, states, dq, rr, active, nactive);
     STG_CUDA(cudaGetLastError());
     return STG_OK;
 }
 
-stg_status launch_xpay_m(int pd, int vh, const char *r, char *d, size_t sr, size_t sd,
-                         const CGState *states, const int *active, const int *nactive, int nslots,
-                         cudaStream_t s)
+stg_status launch_xpay_m(int pd, int vh, const char *r, char *d, size_t sr, size_t sd, CGState *states,
+                         const double *rr, const int *active, const int *nactive, int nslots, cudaStream_t s)
 {
-    const dim3 grid(grid_vec(vh, pr_of(pd)), nslots);
-    if (pd == P64) k_xpay_m<P64, P64><<<grid, kBlock, 0, s>>>(vh, r, d, sr, sd, states, active, nactive);
-    else if (pd == P32) k_xpay_m<P32, P32><<<grid, kBlock, 0, s>>>(vh, r, d, sr, sd, states, active, nactive);
-    else if (pd == P16) k_xpay_m<P16, P32><<<grid, kBlock, 0, s>>>(vh, r, d, sr, sd, states, active, nactive);
-    else if (pd == PB16) k_xpay_m<PB16, P32><<<grid, kBlock, 0, s>>>(vh, r, d, sr, sd, states, active, nactive);
-    else k_xpay_m<PX16, P32><<<grid, kBlock, 0, s>>>(vh, r, d, sr, sd, states, active, nactive);
+    const dim3 grid(grid_vec(vh, nslots), nslots);
+    STG_DISPATCH_PD(pd, k_xpay_m, vh, r, d, sr, sd, states, rr, active, nactive);
     STG_CUDA(cudaGetLastError());
     return STG_OK;
 }

@@ -20,7 +20,7 @@
 //   EPI_GATE  out = D in, skipped when the CG state flag is raised
 //   EPI_A     out = m^2 w - D in                     (w = the even input d)
 //   EPI_A_DOT as EPI_A, plus Re sum w^dag out in FP64 -> *dot
-//   EPI_A_CG  as EPI_A_DOT inside CG: alpha = delta / d^dag A d -> state
+//   EPI_A_CG  as EPI_A inside CG, with block partials of Re sum w^dag out
 //   EPI_RES   out = w - m^2 v + D in = b - A x, plus |out|^2 in FP64 -> *dot
 #include "dslash_site.cuh"
 
@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const Dslas
     pdl_trigger();
     if (EPI == EPI_A_CG || EPI == EPI_GATE) {
         if (a.state->flag != FLAG_RUN) return;  // uniform over the grid
+        if (EPI == EPI_GATE && blockIdx.x == 0 && threadIdx.x == 0) cg_commit(a.state);
     }
     const int i = blockIdx.x * kBlock + threadIdx.x;
     const int vh = a.g.Vh;
@@ -76,25 +77,15 @@ __global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const Dslas
             for (int c = 0; c < 3; ++c) dot += d.r[c] * os.r[c] + d.i[c] * os.i[c];
         }
     }
-    if (EPI == EPI_A_DOT || EPI == EPI_A_CG || EPI == EPI_RES) {
+    if constexpr (EPI == EPI_A_CG) {
+        if constexpr (P == P64) publish_partial<kBlock>(double(dot), a.state, a.partials);
+        else publish_partial<kBlock>(FF{float(dot), 0.f}, a.state, a.partials);
+    } else if constexpr (EPI == EPI_A_DOT || EPI == EPI_RES) {
         double total;
         bool last;
-        if constexpr (P == P64) {
-            last = grid_sum<kBlock>(double(dot), a.partials, a.counter, total);
-        } else {
-            FF v;
-            v.hi = float(dot);
-            v.lo = 0.f;
-            last = grid_sum_ff<kBlock>(v, reinterpret_cast<float2 *>(a.partials), a.counter, total);
-        }
-        if (last) {
-            if (EPI == EPI_A_CG) {
-                CGState *st = a.state;
-                set_alpha(st, total);
-            } else {
-                *a.dot = total;
-            }
-        }
+        if constexpr (P == P64) last = grid_sum<kBlock>(double(dot), a.partials, a.counter, total);
+        else last = grid_sum_ff<kBlock>(FF{float(dot), 0.f}, reinterpret_cast<float2 *>(a.partials), a.counter, total);
+        if (last) *a.dot = total;
     }
 }
 

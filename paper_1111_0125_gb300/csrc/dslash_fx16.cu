@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(kBlock, STG_FX2_MINBLOCKS) k_dslash_fx2(const 
     pdl_trigger();
     if (EPI == EPI_A_CG || EPI == EPI_GATE) {
         if (a.state->flag != FLAG_RUN) return;  // uniform over the grid
+        if (EPI == EPI_GATE && blockIdx.x == 0 && threadIdx.x == 0) cg_commit(a.state);
     }
     const int vh = a.g.Vh;
     const int iA = blockIdx.x * (2 * kBlock) + threadIdx.x;
@@ -171,16 +172,11 @@ __global__ void __launch_bounds__(kBlock, STG_FX2_MINBLOCKS) k_dslash_fx2(const 
         dot.hi = dA_B.x;
         dot = ff_add(dot, FF{dA_B.y, 0.f});
     }
-    if (EPI == EPI_A_DOT || EPI == EPI_A_CG || EPI == EPI_RES) {
+    if (EPI == EPI_A_CG) {
+        publish_partial<kBlock>(dot, a.state, a.partials);
+    } else if (EPI == EPI_A_DOT || EPI == EPI_RES) {
         double total;
-        if (grid_sum_ff<kBlock>(dot, reinterpret_cast<float2 *>(a.partials), a.counter, total)) {
-            if (EPI == EPI_A_CG) {
-                CGState *st = a.state;
-                set_alpha(st, total);
-            } else {
-                *a.dot = total;
-            }
-        }
+        if (grid_sum_ff<kBlock>(dot, reinterpret_cast<float2 *>(a.partials), a.counter, total)) *a.dot = total;
     }
 }
 
@@ -200,8 +196,8 @@ __global__ void __launch_bounds__(kBlock, STG_FX2_MINBLOCKS) k_dslash_fx2(const 
 // the register-fed kernel.
 //
 // Each wait on an mbarrier gives up after about a second: it counts the
-// event in g_fx_wait_timeouts, the CG state gets FLAG_TIMEOUT (directly, or
-// through a NaN grid sum), and the CTA lets its own copies land before it
+// event in g_fx_wait_timeouts, the CG state gets FLAG_TIMEOUT (outside CG the
+// grid sum becomes NaN), and the CTA lets its own copies land before it
 // exits.
 // ---------------------------------------------------------------------------
 constexpr int kFxCons = kFxTile / 2;       // threads, two sites each
@@ -236,9 +232,9 @@ __global__ void __launch_bounds__(kFxCons, kFxCtasPerSM) k_dslash_fx2_staged(con
     const int ntiles = (vh + kFxTile - 1) / kFxTile;
     const int c = threadIdx.x, lane = c & 31;
     // Before the wait only kernels two or more back have completed (the
-    // predecessor triggers after its own wait); the flag's writer is one of
-    // them, except for a timeout, so this read only decides whether to
-    // prefetch and the check after the wait decides.
+    // predecessor triggers after its own wait) and the predecessor may be the
+    // flag's writer, so this read only decides whether to prefetch and the
+    // check after the wait decides.
     const bool prefetch = (EPI != EPI_A_CG && EPI != EPI_GATE) ||
                           *(volatile const int *)&a.state->flag == FLAG_RUN;
     // the (tile, mu) items of this CTA in order, item q = 4 j + mu, go
@@ -277,6 +273,7 @@ __global__ void __launch_bounds__(kFxCons, kFxCtasPerSM) k_dslash_fx2_staged(con
             }
             return;
         }
+        if (EPI == EPI_GATE && blockIdx.x == 0 && c == 0) cg_commit(a.state);
         if (!prefetch && c == 0) {  // the flag was lowered after the early read
 #pragma unroll
             for (int q = 0; q < kFxStages; ++q) {
@@ -396,23 +393,13 @@ __global__ void __launch_bounds__(kFxCons, kFxCtasPerSM) k_dslash_fx2_staged(con
 #pragma unroll
         for (int q = 0; q < kFxStages; ++q)
             if (issued[q]) mbar_wait(smem_addr(&full[q]), (issued[q] - 1u) & 1u, nullptr, &g_fx_wait_timeouts);
-        if (EPI == EPI_GATE) a.state->flag = FLAG_TIMEOUT;  // no grid sum here
+        if (EPI == EPI_GATE || EPI == EPI_A_CG) a.state->flag = FLAG_TIMEOUT;
     }
-    if (EPI == EPI_A_DOT || EPI == EPI_A_CG || EPI == EPI_RES) {
+    if (EPI == EPI_A_CG) {
+        publish_partial<kFxCons>(dot, a.state, a.partials);
+    } else if (EPI == EPI_A_DOT || EPI == EPI_RES) {
         double total;
-        if (grid_sum_ff<kFxCons>(dot, reinterpret_cast<float2 *>(a.partials), a.counter, total)) {
-            if (EPI == EPI_A_CG) {
-                CGState *st = a.state;
-                if (!isfinite(total) && *(volatile unsigned *)&g_fx_wait_timeouts) {
-                    st->pAp = total;
-                    st->flag = FLAG_TIMEOUT;
-                } else {
-                    set_alpha(st, total);
-                }
-            } else {
-                *a.dot = total;
-            }
-        }
+        if (grid_sum_ff<kFxCons>(dot, reinterpret_cast<float2 *>(a.partials), a.counter, total)) *a.dot = total;
     }
 }
 

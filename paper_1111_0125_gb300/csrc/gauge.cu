@@ -551,7 +551,8 @@ stg_status workspace_get(stg_gauge *g, Workspace **out)
         return STG_ERR_OOM;
     }
     ws->n_partials = (size_t)((g->geom.Vh + kBlock - 1) / kBlock) + 64;
-    cudaError_t e = cudaMalloc((void **)&ws->partials, ws->n_partials * sizeof(double));
+    cudaError_t e = cudaMalloc((void **)&ws->partials, (ws->n_partials + kRrPartials) * sizeof(double));
+    ws->rr = ws->partials + ws->n_partials;
     if (e == cudaSuccess) e = cudaMalloc((void **)&ws->state, sizeof(CGState));
     if (e == cudaSuccess) e = cudaMemset(ws->state, 0, sizeof(CGState));
     if (e == cudaSuccess) e = cudaMallocHost((void **)&ws->state_host, sizeof(CGState));

@@ -261,7 +261,7 @@ void mrhs_free(MrhsWs *m)
     if (!m) return;
     if (m->graph) cudaGraphExecDestroy(m->graph);
     void *v[] = {m->x64, m->b64, m->r64, m->y, m->r, m->d, m->q, m->t, m->partials, m->states,
-                 m->active, m->counter, m->tmp};
+                 m->active, m->tmp};
     for (void *p : v) cudaFree(p);
     if (m->states_host) cudaFreeHost(m->states_host);
     if (m->active_host) cudaFreeHost(m->active_host);
@@ -291,7 +291,7 @@ static stg_status mrhs_alloc(const stg_gauge *g, int n, int pd, MrhsWs **out)
     m->f64 = vh * 48;
     m->fr = vh * field_site_bytes(pr_of_m(pd));
     m->fd = vh * field_site_bytes(pd);
-    m->pstride = (size_t)((g->geom.Vh + 127) / 128) + 1024;  // >= both grids of the iteration
+    m->pstride = (size_t)((g->geom.Vh + 127) / 128) + 1024;  // kDqPartials + kRrPartials, and the FP64 residual's grid
     stg_status st = STG_OK;
     char **bufs[] = {&m->x64, &m->b64, &m->r64};
     for (char **b : bufs)
@@ -305,10 +305,8 @@ static stg_status mrhs_alloc(const stg_gauge *g, int n, int pd, MrhsWs **out)
     if (st == STG_OK) st = dev_alloc((void **)&m->partials, n * m->pstride * sizeof(double));
     if (st == STG_OK) st = dev_alloc((void **)&m->states, n * sizeof(CGState));
     if (st == STG_OK) st = dev_alloc((void **)&m->active, (n + 1) * sizeof(int));
-    if (st == STG_OK) st = dev_alloc((void **)&m->counter, 256);
     if (st == STG_OK) {
         cudaError_t e = cudaMemset(m->states, 0, n * sizeof(CGState));
-        if (e == cudaSuccess) e = cudaMemset(m->counter, 0, 256);
         if (e == cudaSuccess) e = cudaMemset(m->active, 0, (n + 1) * sizeof(int));
         if (e == cudaSuccess) e = cudaMallocHost((void **)&m->states_host, n * sizeof(CGState));
         if (e == cudaSuccess) e = cudaMallocHost((void **)&m->active_host, (n + 1) * sizeof(int));
@@ -334,7 +332,6 @@ static stg_status iteration_m(const stg_gauge *g, MrhsWs *m, const LinkField *lf
     a.active = m->active + 1;
     a.states = m->states;
     a.partials = reinterpret_cast<float2 *>(m->partials);
-    a.counter = m->counter;
     a.parity = 1;
     a.in = m->d;
     a.out = m->t;
@@ -345,9 +342,10 @@ static stg_status iteration_m(const stg_gauge *g, MrhsWs *m, const LinkField *lf
     a.w = m->d;
     STG_TRY(launch_m(g, lf, m->shape, EPI_A_CG, a, s));
     const int vh = g->geom.Vh;
-    STG_TRY(launch_update_m(m->pd, vh, m->y, m->r, m->d, m->q, m->fr, m->fd, m->states, m->partials,
-                            m->pstride, m->active + 1, m->active, m->nrhs, s));
-    return launch_xpay_m(m->pd, vh, m->r, m->d, m->fr, m->fd, m->states, m->active + 1, m->active,
+    double *rr = m->partials + (size_t)m->nrhs * kDqPartials;
+    STG_TRY(launch_update_m(m->pd, vh, m->y, m->r, m->d, m->q, m->fr, m->fd, m->states, m->partials, rr,
+                            m->active + 1, m->active, m->nrhs, s));
+    return launch_xpay_m(m->pd, vh, m->r, m->d, m->fr, m->fd, m->states, rr, m->active + 1, m->active,
                          m->nrhs, s);
 }
 

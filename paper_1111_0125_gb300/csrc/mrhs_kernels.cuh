@@ -13,8 +13,8 @@
 // nactive) so that the host can drop converged systems between chunks
 // without recapturing the CUDA graph; inside a chunk the per-system CG flag
 // is checked as well.  The fused epilogue reduces d_k^dag q_k per system in
-// compensated FP32 pairs (block partials per system, last block finishes all
-// systems in a fixed order).
+// compensated FP32 pairs to one partial per block and system, which the update
+// kernel adds up.
 #pragma once
 
 #include <stdlib.h>
@@ -40,7 +40,6 @@ struct MrhsArgs {
     CGState *states;       // per system (EPI_GATE, EPI_A_CG)
     float m2[kMaxRhs];     // EPI_A: m_k^2
     float2 *partials;      // EPI_A_CG: [nrhs][gridDim.x]
-    unsigned *counter;     // EPI_A_CG: arrival counter
     int grid_cap;          // blocks launched at most (they stride over site tiles)
     int grid_limit;        // staged kernels: at most this many CTAs (0 = all resident;
                            // STG_MRHS_GRID, read per call, for tests)
@@ -48,6 +47,24 @@ struct MrhsArgs {
 };
 
 constexpr int kMrhsBlock = 256;
+// blocks of an EPI_A_CG launch at most: their partials share an array with
+// the update's
+constexpr int kDqPartials = 640;
+static_assert(kDqPartials + kRrPartials <= 1024, "the session's partials per system");
+
+// EPI_GATE, block 0: the iteration's scalars of every listed system
+__device__ __forceinline__ void commit_systems(const MrhsArgs &a, int nact)
+{
+    if (blockIdx.x == 0)
+        for (int kk = threadIdx.x; kk < nact; kk += blockDim.x) cg_commit(a.states + (a.active ? a.active[kk] : kk));
+}
+
+// EPI_A_CG: this block's partial of system k
+__device__ __forceinline__ void publish_system(const MrhsArgs &a, int k, FF sum)
+{
+    a.partials[(size_t)k * gridDim.x + blockIdx.x] = make_float2(sum.hi, sum.lo);
+    if (blockIdx.x == 0) a.states[k].n_part = (int)gridDim.x;
+}
 
 // TPS threads share one site (consecutive lanes of a warp): they load the
 // same link words, which the load unit merges into one request, so the
@@ -65,6 +82,7 @@ __global__ void __launch_bounds__(kMrhsBlock) k_dslash_m(const MrhsArgs a)
     constexpr int kTile = BS / TPS;          // sites per tile
     const int ntiles = (vh + kTile - 1) / kTile;
 
+    if (EPI == EPI_GATE) commit_systems(a, nact);
     __shared__ float2 red[NB][TPS][BS / 32];
     __shared__ FF sys_acc[kMaxRhs];          // this block's d^dag q per list slot
     if (EPI == EPI_A_CG) {
@@ -192,49 +210,8 @@ __global__ void __launch_bounds__(kMrhsBlock) k_dslash_m(const MrhsArgs a)
     }
     }  // tiles
 
-    if (EPI == EPI_A_CG) {
-        for (int kk = threadIdx.x; kk < nact; kk += BS) {
-            const int k = a.active ? a.active[kk] : kk;
-            a.partials[(size_t)k * gridDim.x + blockIdx.x] = make_float2(sys_acc[kk].hi, sys_acc[kk].lo);
-        }
-        __threadfence();
-        __syncthreads();
-    }
-
-    if (EPI == EPI_A_CG) {
-        __shared__ int is_last;
-        if (threadIdx.x == 0) {
-            __threadfence();
-            const unsigned ticket = atomicAdd(a.counter, 1u);
-            is_last = (ticket == gridDim.x - 1);
-        }
-        __syncthreads();
-        if (!is_last) return;
-        __threadfence();
-        // one warp per system (fixed summation order per system)
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        for (int kk = w; kk < nact; kk += BS / 32) {
-            const int k = a.active ? a.active[kk] : kk;
-            if (a.states[k].flag != FLAG_RUN) continue;  // uniform in the warp
-            FF acc = {0.f, 0.f};
-            for (int b = lane; b < (int)gridDim.x; b += 32) {
-                const float2 p = __ldcg(a.partials + (size_t)k * gridDim.x + b);
-                FF t;
-                t.hi = p.x;
-                t.lo = p.y;
-                acc = ff_add(acc, t);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc = ff_add(acc, ff_shfl_down(acc, o));
-            if (lane == 0) {
-                CGState *st = a.states + k;
-                const double total = (double)acc.hi + (double)acc.lo;
-                set_alpha(st, total);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) *a.counter = 0u;
-    }
+    if (EPI == EPI_A_CG)
+        for (int kk = threadIdx.x; kk < nact; kk += BS) publish_system(a, a.active ? a.active[kk] : kk, sys_acc[kk]);
 }
 
 // ---------------------------------------------------------------------------
@@ -517,6 +494,7 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
             }
         }
     }
+    if (EPI == EPI_GATE) commit_systems(a, nact);
     if (EPI == EPI_A_CG)
         for (int k = threadIdx.x; k < kMsWarps * kMaxRhs; k += kMsThreads)
             sysw[k / kMaxRhs][k % kMaxRhs].hi = sysw[k / kMaxRhs][k % kMaxRhs].lo = 0.f;
@@ -790,49 +768,10 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
             FF sum = sysw[0][kk];
 #pragma unroll
             for (int w = 1; w < kMsWarps; ++w) sum = ff_add(sum, sysw[w][kk]);
-            if (abort_flag) sum.hi = __int_as_float(0x7fc00000);  // the system's sum becomes NaN
-            const int k = a.active ? a.active[kk] : kk;
-            a.partials[(size_t)k * gridDim.x + blockIdx.x] = make_float2(sum.hi, sum.lo);
+            publish_system(a, a.active ? a.active[kk] : kk, sum);
         }
-        __threadfence();
-        __syncthreads();
-        __shared__ int is_last;
-        if (threadIdx.x == 0) {
-            __threadfence();
-            const unsigned ticket = atomicAdd(a.counter, 1u);
-            is_last = (ticket == gridDim.x - 1);
-        }
-        __syncthreads();
-        if (!is_last) return;
-        __threadfence();
-        // one warp per system (fixed summation order per system)
-        for (int kk = warp; kk < nact; kk += kMsWarps) {
-            const int k = a.active ? a.active[kk] : kk;
-            if (a.states[k].flag != FLAG_RUN) continue;  // uniform in the warp
-            FF acc = {0.f, 0.f};
-            for (int b = lane; b < (int)gridDim.x; b += 32) {
-                const float2 p = __ldcg(a.partials + (size_t)k * gridDim.x + b);
-                FF t;
-                t.hi = p.x;
-                t.lo = p.y;
-                acc = ff_add(acc, t);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc = ff_add(acc, ff_shfl_down(acc, o));
-            if (lane == 0) {
-                CGState *st = a.states + k;
-                const double total = (double)acc.hi + (double)acc.lo;
-                if (!isfinite(total) && *(volatile unsigned *)&g_ms_wait_timeouts) {
-                    st->pAp = total;
-                    st->flag = FLAG_TIMEOUT;
-                } else {
-                    set_alpha(st, total);
-                }
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) *a.counter = 0u;
-    } else if (EPI == EPI_GATE) {
+    }
+    if (EPI == EPI_A_CG || EPI == EPI_GATE) {
         if (threadIdx.x == 0 && abort_flag)
             for (int kk = 0; kk < nact; ++kk) a.states[a.active ? a.active[kk] : kk].flag = FLAG_TIMEOUT;
     }
@@ -863,7 +802,7 @@ void launch_ms_nb(int epi, const MrhsArgs &a, cudaStream_t s)
         return sms * per_sm;
     }();
     const int ntiles = (a.g.Vh + kMTile - 1) / kMTile;
-    int cap = resident;
+    int cap = resident < kDqPartials ? resident : kDqPartials;
     if (a.grid_limit > 0 && a.grid_limit < cap) cap = a.grid_limit;
     const int grid = ntiles < cap ? ntiles : cap;
     switch (epi) {

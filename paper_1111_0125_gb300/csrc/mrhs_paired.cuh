@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(kMspThreads, NB == 2 ? 4 : 3) k_dslash_msp(con
             }
         }
     }
+    if (EPI == EPI_GATE) commit_systems(a, nact);
     if (EPI == EPI_A_CG)
         for (int k = threadIdx.x; k < kMspWarps * kMaxRhs; k += kMspThreads)
             sysw[k / kMaxRhs][k % kMaxRhs] = FF{0.f, 0.f};
@@ -211,46 +212,10 @@ __global__ void __launch_bounds__(kMspThreads, NB == 2 ? 4 : 3) k_dslash_msp(con
             FF sum = sysw[0][kk];
 #pragma unroll
             for (int w = 1; w < kMspWarps; ++w) sum = ff_add(sum, sysw[w][kk]);
-            if (abort_flag) sum.hi = __int_as_float(0x7fc00000);  // the system's sum becomes NaN
-            const int k = a.active ? a.active[kk] : kk;
-            a.partials[(size_t)k * gridDim.x + blockIdx.x] = make_float2(sum.hi, sum.lo);
+            publish_system(a, a.active ? a.active[kk] : kk, sum);
         }
-        __threadfence();
-        __syncthreads();
-        __shared__ int is_last;
-        if (threadIdx.x == 0) {
-            __threadfence();
-            const unsigned ticket = atomicAdd(a.counter, 1u);
-            is_last = (ticket == gridDim.x - 1);
-        }
-        __syncthreads();
-        if (!is_last) return;
-        __threadfence();
-        // one warp per system (fixed summation order per system)
-        for (int kk = grp; kk < nact; kk += kMspWarps) {
-            const int k = a.active ? a.active[kk] : kk;
-            if (a.states[k].flag != FLAG_RUN) continue;  // uniform in the warp
-            FF acc = {0.f, 0.f};
-            for (int b = lane; b < (int)gridDim.x; b += 32) {
-                const float2 p = __ldcg(a.partials + (size_t)k * gridDim.x + b);
-                acc = ff_add(acc, FF{p.x, p.y});
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc = ff_add(acc, ff_shfl_down(acc, o));
-            if (lane == 0) {
-                CGState *st = a.states + k;
-                const double total = (double)acc.hi + (double)acc.lo;
-                if (!isfinite(total) && *(volatile unsigned *)&g_msp_wait_timeouts) {
-                    st->pAp = total;
-                    st->flag = FLAG_TIMEOUT;
-                } else {
-                    set_alpha(st, total);
-                }
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) *a.counter = 0u;
-    } else if (EPI == EPI_GATE) {
+    }
+    if (EPI == EPI_A_CG || EPI == EPI_GATE) {
         if (threadIdx.x == 0 && abort_flag)
             for (int kk = 0; kk < nact; ++kk) a.states[a.active ? a.active[kk] : kk].flag = FLAG_TIMEOUT;
     }
@@ -277,7 +242,7 @@ void launch_msp_nb(int epi, const MrhsArgs &a, cudaStream_t s)
         return sms * per_sm;
     }();
     const int ntiles = (a.g.Vh + kMTile - 1) / kMTile;
-    int cap = resident;
+    int cap = resident < kDqPartials ? resident : kDqPartials;
     if (a.grid_limit > 0 && a.grid_limit < cap) cap = a.grid_limit;
     const int grid = ntiles < cap ? ntiles : cap;
     switch (epi) {

@@ -718,6 +718,7 @@ struct CGState {
     double delta_old;
     double pAp;        // d^dag A d
     double alpha, beta;
+    double c_delta, c_rmax2;  // delta_new and rmax2 at the start of the iteration (cg_commit)
     double rmax2;      // largest |r|^2 since the last update (or at reset)
     double stop_r2;    // tol^2 |b|^2: iterated-residual stopping point
     double trig2;      // delta^2: reliable-update trigger (0 = never)
@@ -725,12 +726,24 @@ struct CGState {
     double result;     // slot for stand-alone reductions
     long long iter;        // iterations done (all precisions)
     long long iter_limit;  // stop when iter reaches this
+    long long c_iter;      // iter at the start of the iteration (cg_commit)
     int flag;
     int track_max;     // 1: rmax2 follows the running maximum (Sec. 3.2)
     unsigned counter;  // arrival counter of the last-block reduction
-    unsigned pad;
+    int n_part;        // block partials of d^dag q that the update adds up
 };
 
+// The scalars of an iteration without a last-block election.  The kernel that
+// needs a grid total adds up the producer's block partials itself, every block
+// the same ones in the same order, while its first operands load: an election
+// (store, fence, atomic, partials back from L2) costs the producer 3 us after
+// its last block, an ordinary launch boundary later the partials cost 1 us.
+//   A's second half-pass    -> partials of d^dag q
+//   update: alpha from them -> partials of |r|^2
+//   xpay: beta, stop tests  -> the state (its block 0)
+// Blocks of one kernel may start after its block 0 has written, so update and
+// xpay read the c_ copies, which block 0 of the next iteration's first
+// half-pass takes (nothing in that kernel reads them).
 // alpha = delta / d^dag A d (Fig. 1), with a breakdown test.  For the exact
 // operator d^dag A d >= m^2 |d|^2, and |d|^2 >= |r|^2 = delta because d = r +
 // beta d_old with d_old orthogonal to r, so alpha <= 1 / m^2.  A
@@ -738,12 +751,25 @@ struct CGState {
 // means the low-precision iteration has lost the operator's positivity: the
 // flag makes the solver take a reliable update and restart from the true
 // residual before y is spoiled by the step.
+__device__ __forceinline__ bool cg_alpha(double delta, double pAp, double m2, double &alpha)
+{
+    alpha = delta / pAp;
+    return pAp > 0.0 && isfinite(pAp) && alpha * m2 <= 16.0;
+}
+
 __device__ __forceinline__ void set_alpha(CGState *st, double pAp)
 {
     st->pAp = pAp;
-    const double alpha = st->delta_new / pAp;
-    if (!(pAp > 0.0) || !isfinite(pAp) || !(alpha * st->m2 <= 16.0)) st->flag = FLAG_BREAKDOWN;
-    else st->alpha = alpha;
+    double alpha;
+    if (cg_alpha(st->delta_new, pAp, st->m2, alpha)) st->alpha = alpha;
+    else st->flag = FLAG_BREAKDOWN;
+}
+
+__device__ __forceinline__ void cg_commit(CGState *st)
+{
+    st->c_delta = st->delta_new;
+    st->c_rmax2 = st->rmax2;
+    st->c_iter = st->iter;
 }
 
 // ---------------------------------------------------------------------------
@@ -834,9 +860,54 @@ __device__ __forceinline__ FF block_sum_ff(FF v, float2 *sm)
             s.lo = sm[lane].y;
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s = ff_add(s, ff_shfl_down(s, o));
+        for (int o = BS / 64; o > 0; o >>= 1) s = ff_add(s, ff_shfl_down(s, o));
     }
     return s;  // valid in thread 0
+}
+
+// One block's partial of d^dag q, and the partials' number, for the update.
+template <int BS>
+__device__ __forceinline__ void publish_partial(FF v, CGState *st, double *partials)
+{
+    __shared__ float2 smf[32];
+    const FF s = block_sum_ff<BS>(v, smf);
+    if (threadIdx.x == 0) {
+        reinterpret_cast<float2 *>(partials)[blockIdx.x] = make_float2(s.hi, s.lo);
+        if (blockIdx.x == 0) st->n_part = (int)gridDim.x;
+    }
+}
+
+template <int BS>
+__device__ __forceinline__ void publish_partial(double v, CGState *st, double *partials)
+{
+    __shared__ double sm[BS];
+    const double s = block_sum_smem<BS>(v, sm);
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = s;
+        if (blockIdx.x == 0) st->n_part = (int)gridDim.x;
+    }
+}
+
+// The sum of n block partials (doubles, or FP32 pairs), in thread 0 of every
+// block that calls it, in one order.
+template <int BS, bool PAIRS>
+__device__ __forceinline__ double sum_partials(const double *partials, int n)
+{
+    if constexpr (PAIRS) {
+        __shared__ float2 smf[32];
+        FF acc = {0.f, 0.f};
+        for (int k = threadIdx.x; k < n; k += BS) {
+            const float2 p = __ldcg(reinterpret_cast<const float2 *>(partials) + k);
+            acc = ff_add(acc, FF{p.x, p.y});
+        }
+        const FF t = block_sum_ff<BS>(acc, smf);
+        return (double)t.hi + (double)t.lo;
+    } else {
+        __shared__ double sm[BS];
+        double acc = 0.0;
+        for (int k = threadIdx.x; k < n; k += BS) acc += __ldcg(partials + k);
+        return block_sum_smem<BS>(acc, sm);
+    }
 }
 
 template <int BS>

@@ -81,7 +81,6 @@ struct MrhsWs {
     double *partials = nullptr;
     CGState *states = nullptr, *states_host = nullptr;
     int *active = nullptr, *active_host = nullptr;  // [0] = count, [1..] = systems
-    unsigned *counter = nullptr;
     void *tmp = nullptr;
     cudaGraphExec_t graph = nullptr;
     int graph_iters = 0;
@@ -137,6 +136,7 @@ stg_status links_fix(const Geom &g, LinkField *lf, cudaStream_t s);
 // Reduction scratch: partial sums (one double per block) and the state.
 struct Workspace {
     double *partials = nullptr;
+    double *rr = nullptr;          // kRrPartials more behind them: |r|^2 of the update
     size_t n_partials = 0;
     CGState *state = nullptr;      // device
     CGState *state_host = nullptr; // pinned mirror for read-back
@@ -210,13 +210,14 @@ int grid_for(long n);
 int num_sms();  // of the device current at the first call
 
 // vector-kernel helpers with explicit operands (cg.cu)
-int vec_grid(long n, int pd);
+// dq: A's block partials of d^dag q, system k's at k times their number per
+// system (CGState::n_part); rr: room for kRrPartials doubles a system
+constexpr int kRrPartials = 384;
 stg_status launch_update_m(int pd, int vh, char *y, char *r, const char *d, const char *q, size_t sr,
-                           size_t sd, CGState *states, double *partials, size_t pstride,
-                           const int *active, const int *nactive, int nslots, cudaStream_t s);
-stg_status launch_xpay_m(int pd, int vh, const char *r, char *d, size_t sr, size_t sd,
-                         const CGState *states, const int *active, const int *nactive, int nslots,
-                         cudaStream_t s);
+                           size_t sd, CGState *states, const double *dq, double *rr, const int *active,
+                           const int *nactive, int nslots, cudaStream_t s);
+stg_status launch_xpay_m(int pd, int vh, const char *r, char *d, size_t sr, size_t sd, CGState *states,
+                         const double *rr, const int *active, const int *nactive, int nslots, cudaStream_t s);
 stg_status launch_reset(int pd, int vh, void *y, void *r, void *d, const void *r64, double beta,
                         int copy_r, cudaStream_t s);
 stg_status launch_accumulate_x(int pr, int vh, void *x64, const void *y, cudaStream_t s);
