@@ -98,17 +98,22 @@ __device__ __forceinline__ void cg_update_body(int vh, void *y, void *r, const v
     fetch();
     __shared__ T sm_alpha;
     __shared__ int sm_ok;
-    const double pAp = sum_partials<kBlock, PD != P64>(dq, st->n_part);
-    if (threadIdx.x == 0) {
-        double a;
-        sm_ok = cg_alpha(st->c_delta, pAp, st->m2, a);
-        sm_alpha = T(a);
-        if (blockIdx.x == 0) {
-            st->pAp = pAp;
-            if (sm_ok) st->alpha = a;
-            else st->flag = FLAG_BREAKDOWN;
+    if constexpr (PD == P64) {
+        const double pAp = sum_partials<kBlock>(dq, st->n_part);
+        if (threadIdx.x == 0) {
+            double a;
+            sm_ok = cg_alpha(st->c_delta, pAp, st->m2, a);
+            sm_alpha = T(a);
+        }
+    } else {
+        const FF pAp = sum_partials_ff<kBlock>(dq, st->n_part);
+        if (threadIdx.x == 0) {
+            float a;
+            sm_ok = ff_alpha(ff_of(st->cf_delta), pAp, st->m2f, a);
+            sm_alpha = T(a);
         }
     }
+    if (threadIdx.x == 0 && blockIdx.x == 0 && !sm_ok) st->flag = FLAG_BREAKDOWN;
     __syncthreads();
     if (!sm_ok) return;
     const T alpha = sm_alpha;
@@ -197,25 +202,43 @@ __device__ __forceinline__ void xpay_body(int vh, const void *r, void *d, CGStat
     fetch();
     __shared__ T sm_beta;
     __shared__ int sm_run;
-    const double total = sum_partials<kBlock, PR != P64>(rr, gridDim.x);
-    if (threadIdx.x == 0) {
-        const double old = st->c_delta;
-        const double beta = total / old;
-        const long long iter = st->c_iter + 1;
-        int flag = FLAG_RUN;
-        if (!isfinite(total)) flag = FLAG_BREAKDOWN;
-        else if (total <= st->stop_r2) flag = FLAG_CONVERGED;
-        else if (st->trig2 > 0.0 && total < st->trig2 * st->c_rmax2) flag = FLAG_UPDATE;
-        else if (iter >= st->iter_limit) flag = FLAG_MAXITER;
-        sm_beta = T(beta);
-        sm_run = flag == FLAG_RUN;
-        if (blockIdx.x == 0) {
-            st->delta_old = old;
-            st->delta_new = total;
-            st->beta = beta;
-            st->iter = iter;
-            if (st->track_max && total > st->c_rmax2) st->rmax2 = total;
-            if (flag != FLAG_RUN) st->flag = flag;
+    if constexpr (PR == P64) {
+        const double total = sum_partials<kBlock>(rr, gridDim.x);
+        if (threadIdx.x == 0) {
+            const double old = st->c_delta;
+            int flag = FLAG_RUN;
+            if (!isfinite(total)) flag = FLAG_BREAKDOWN;
+            else if (total <= st->stop_r2) flag = FLAG_CONVERGED;
+            else if (st->trig2 > 0.0 && total < st->trig2 * st->c_rmax2) flag = FLAG_UPDATE;
+            else if (st->c_iter + 1 >= st->iter_limit) flag = FLAG_MAXITER;
+            sm_beta = T(total / old);
+            sm_run = flag == FLAG_RUN;
+            if (blockIdx.x == 0) {
+                st->delta_old = old;
+                st->delta_new = total;
+                if (st->track_max && total > st->c_rmax2) st->rmax2 = total;
+                st->iter = st->c_iter + 1;
+                if (flag != FLAG_RUN) st->flag = flag;
+            }
+        }
+    } else {
+        const FF total = sum_partials_ff<kBlock>(rr, gridDim.x);
+        if (threadIdx.x == 0) {
+            const FF old = ff_of(st->cf_delta), top = ff_of(st->cf_rmax2);
+            int flag = FLAG_RUN;
+            if (!isfinite(total.hi)) flag = FLAG_BREAKDOWN;
+            else if (ff_le(total, ff_of(st->f_stop))) flag = FLAG_CONVERGED;
+            else if (st->trig2f > 0.f && ff_less(total, ff_scale(top, st->trig2f))) flag = FLAG_UPDATE;
+            else if (st->c_iter + 1 >= st->iter_limit) flag = FLAG_MAXITER;
+            sm_beta = T(ff_div(total, old));
+            sm_run = flag == FLAG_RUN;
+            if (blockIdx.x == 0) {
+                st->f_delta_old = make_float2(old.hi, old.lo);
+                st->f_delta = make_float2(total.hi, total.lo);
+                if (st->track_max && ff_less(top, total)) st->f_rmax2 = make_float2(total.hi, total.lo);
+                st->iter = st->c_iter + 1;
+                if (flag != FLAG_RUN) st->flag = flag;
+            }
         }
     }
     __syncthreads();
@@ -595,11 +618,13 @@ static stg_status read_state(Workspace *ws, cudaStream_t s)
 {
     STG_CUDA(cudaMemcpyAsync(ws->state_host, ws->state, sizeof(CGState), cudaMemcpyDeviceToHost, s));
     STG_CUDA(cudaStreamSynchronize(s));
+    state_got(ws->state_host);
     return STG_OK;
 }
 
 static stg_status write_state(Workspace *ws, cudaStream_t s)
 {
+    state_put(ws->state_host, ws->cg_sloppy);
     STG_CUDA(cudaMemcpyAsync(ws->state, ws->state_host, sizeof(CGState), cudaMemcpyHostToDevice, s));
     return STG_OK;
 }

@@ -32,6 +32,10 @@ namespace stg {
 // 193 / 270 us.
 constexpr int min_blocks(int p, int r) { return p == P64 && (r & kFixLinks) ? 2 : 1; }
 
+template <typename T> __device__ __forceinline__ T pick_m2(double d, float f);
+template <> __device__ __forceinline__ double pick_m2<double>(double d, float) { return d; }
+template <> __device__ __forceinline__ float pick_m2<float>(double, float f) { return f; }
+
 template <int P, int R, int EPI>
 __global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const DslashArgs a)
 {
@@ -52,7 +56,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const Dslas
         } else if (EPI == EPI_RES) {
             const Vec3<T> b = FieldIO<P>::load_nc(a.w, vh, i);
             const Vec3<T> x = FieldIO<P>::load_nc(a.v, vh, i);
-            const T m2 = T(a.m2);
+            const T m2 = pick_m2<T>(a.m2, a.m2f);
             Vec3<T> o;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -63,7 +67,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const Dslas
 #pragma unroll
             for (int c = 0; c < 3; ++c) dot += os.r[c] * os.r[c] + os.i[c] * os.i[c];
         } else {
-            const T m2 = (EPI == EPI_A_CG) ? T(a.state->m2) : T(a.m2);
+            const T m2 = (EPI == EPI_A_CG) ? pick_m2<T>(a.state->m2, a.state->m2f) : pick_m2<T>(a.m2, a.m2f);
             const Vec3<T> d = FieldIO<P>::load_nc(a.w, vh, i);
             Vec3<T> o;
 #pragma unroll
@@ -119,6 +123,7 @@ stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &L
     a.w = L.w;
     a.v = L.v;
     a.m2 = L.m2;
+    a.m2f = (float)L.m2;
     a.dot = L.dot;
     a.state = L.state;
     a.partials = L.partials;

@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kBlock, STG_FX2_MINBLOCKS) k_dslash_fx2(const 
             load_field2(a.in, jbA, jbB, v);
             bwd2<12>(u, v, s2b, A);
         }
-        const float m2 = (EPI == EPI_A_CG) ? float(a.state->m2) : float(a.m2);
+        const float m2 = (EPI == EPI_A_CG) ? a.state->m2f : a.m2f;
         f2 dA_B;
         if (EPI == EPI_RES) {
             const f2 k = make_float2(LinkPost<PX16>::k, LinkPost<PX16>::k);
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(kFxCons, kFxCtasPerSM) k_dslash_fx2_staged(con
             dot.hi = __int_as_float(0x7fc00000);  // the grid sum becomes NaN
             break;
         }
-        const float m2 = (EPI == EPI_A_CG) ? float(a.state->m2) : float(a.m2);
+        const float m2 = (EPI == EPI_A_CG) ? a.state->m2f : a.m2f;
         f2 dA_B;
         if (EPI == EPI_RES) {
             const f2 kk = make_float2(LinkPost<P>::k, LinkPost<P>::k);

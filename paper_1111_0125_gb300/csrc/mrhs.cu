@@ -393,7 +393,9 @@ static stg_status sync_states(MrhsWs *m, cudaStream_t s, bool to_host)
     if (to_host) {
         STG_CUDA(cudaMemcpyAsync(m->states_host, m->states, bytes, cudaMemcpyDeviceToHost, s));
         STG_CUDA(cudaStreamSynchronize(s));
+        for (int k = 0; k < m->nrhs; ++k) state_got(m->states_host + k);
     } else {
+        for (int k = 0; k < m->nrhs; ++k) state_put(m->states_host + k, m->pd);
         STG_CUDA(cudaMemcpyAsync(m->states, m->states_host, bytes, cudaMemcpyHostToDevice, s));
     }
     return STG_OK;

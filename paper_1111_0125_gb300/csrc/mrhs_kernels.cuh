@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kMrhsBlock) k_dslash_m(const MrhsArgs a)
                 if (EPI == EPI_NONE || EPI == EPI_GATE) {
                     FieldIO<P>::store(out, vh, i, acc[q]);
                 } else {
-                    const T m2 = (EPI == EPI_A_CG) ? T(a.states[rid[q]].m2) : T(a.m2[rid[q]]);
+                    const T m2 = (EPI == EPI_A_CG) ? a.states[rid[q]].m2f : T(a.m2[rid[q]]);
                     const Vec3<T> d = FieldIO<P>::load_nc(a.w + rid[q] * a.fstride, vh, i);
                     Vec3<T> o;
 #pragma unroll
@@ -713,7 +713,7 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
                 if (EPI == EPI_NONE || EPI == EPI_GATE) {
                     FieldIO<P>::store(out, vh, i, acc[q]);
                 } else {
-                    const T m2 = (EPI == EPI_A_CG) ? T(a.states[rid[q]].m2) : T(a.m2[rid[q]]);
+                    const T m2 = (EPI == EPI_A_CG) ? a.states[rid[q]].m2f : T(a.m2[rid[q]]);
                     const Vec3<T> d = FieldIO<P>::load_nc(a.w + rid[q] * a.fstride, vh, i);
                     Vec3<T> o;
 #pragma unroll

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kMspThreads, NB == 2 ? 4 : 3) k_dslash_msp(con
                         epilogue_pair<EPI_NONE>(out, iA, iB, okA, okB, dr, di, 0.f, make_uint4(0, 0, 0, 0),
                                                 make_uint4(0, 0, 0, 0));
                     } else {
-                        const float m2 = (EPI == EPI_A_CG) ? float(a.states[rid[q]].m2) : a.m2[rid[q]];
+                        const float m2 = (EPI == EPI_A_CG) ? a.states[rid[q]].m2f : a.m2[rid[q]];
                         const uint4 *w = reinterpret_cast<const uint4 *>(a.w + rid[q] * a.fstride);
                         const uint4 wA = __ldg(w + jA), wB = __ldg(w + jB);
                         const f2 d2 = epilogue_pair<EPI_A_DOT>(out, iA, iB, okA, okB, dr, di, m2, wA, wB);

@@ -731,6 +731,11 @@ struct CGState {
     int track_max;     // 1: rmax2 follows the running maximum (Sec. 3.2)
     unsigned counter;  // arrival counter of the last-block reduction
     int n_part;        // block partials of d^dag q that the update adds up
+    // Mixed CG (ff = 1): the scalars as FP32 pairs (hi, lo), which its kernels
+    // use in place of the doubles above; the host converts (state_put, state_got)
+    int ff;
+    float m2f, trig2f;
+    float2 f_stop, f_delta, f_delta_old, f_rmax2, cf_delta, cf_rmax2;
 };
 
 // The scalars of an iteration without a last-block election.  The kernel that
@@ -770,6 +775,8 @@ __device__ __forceinline__ void cg_commit(CGState *st)
     st->c_delta = st->delta_new;
     st->c_rmax2 = st->rmax2;
     st->c_iter = st->iter;
+    st->cf_delta = st->f_delta;
+    st->cf_rmax2 = st->f_rmax2;
 }
 
 // ---------------------------------------------------------------------------
@@ -836,6 +843,56 @@ __device__ __forceinline__ FF ff_add(FF a, FF b)
     return r;
 }
 
+__device__ __forceinline__ FF ff_of(float2 a) { return FF{a.x, a.y}; }
+
+// a < b (a <= b); exact where the pairs are close
+__device__ __forceinline__ bool ff_less(FF a, FF b) { return (a.hi - b.hi) + (a.lo - b.lo) < 0.f; }
+__device__ __forceinline__ bool ff_le(FF a, FF b) { return (a.hi - b.hi) + (a.lo - b.lo) <= 0.f; }
+
+// a / b in FP32 from the pairs' 48 bits: one rounding of a quotient good to
+// 2^-46.  An FP64 division takes 1650 cycles here (its dependent steps run on
+// a pipe of 2 lanes), more than the rest of an iteration's scalars.
+__device__ __forceinline__ float ff_div(FF a, FF b)
+{
+    const float q = a.hi / b.hi;
+    const float r = fmaf(-q, b.hi, a.hi) + fmaf(-q, b.lo, a.lo);
+    return q + r / b.hi;
+}
+
+__device__ __forceinline__ FF ff_scale(FF a, float s)
+{
+    const float p = a.hi * s;
+    return FF{p, fmaf(a.hi, s, -p) + a.lo * s};
+}
+
+// alpha = delta / d^dag q of the mixed CG, with the breakdown test of cg_alpha
+__device__ __forceinline__ bool ff_alpha(FF delta, FF pAp, float m2, float &alpha)
+{
+    alpha = ff_div(delta, pAp);
+    return pAp.hi > 0.f && isfinite(pAp.hi) && alpha * m2 <= 16.f;
+}
+
+// hi + lo as a double by integer operations (FP64 instructions only outside
+// the normal FP32 range): the sum of both significands at 62 bits, rounded to
+// nearest
+__device__ __forceinline__ double ff_double(FF a)
+{
+    const unsigned uh = __float_as_uint(a.hi), ul = __float_as_uint(a.lo);
+    const int eh = (int)((uh >> 23) & 0xffu), el = (int)((ul >> 23) & 0xffu);
+    if (eh == 0 || eh == 255 || el >= eh) return (double)a.hi + (double)a.lo;
+    long long v = (long long)((uh & 0x7fffffu) | 0x800000u) << 38;
+    const int d = eh - el;
+    long long l = (el == 0 || d > 61) ? 0ll : ((long long)((ul & 0x7fffffu) | 0x800000u) << 38) >> d;
+    if ((uh ^ ul) & 0x80000000u) l = -l;
+    v += l;  // positive: |lo| < |hi|
+    const int lz = __clzll(v);
+    const unsigned long long n = (unsigned long long)v << lz;
+    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);
+    // hi = 1.m 2^(eh - 127) has its leading one at bit 61 of v
+    const unsigned long long r = m + ((unsigned long long)(unsigned)(eh - 127 + 1023 + 2 - lz - 1) << 52);
+    return __longlong_as_double((long long)(r | ((unsigned long long)(uh & 0x80000000u) << 32)));
+}
+
 __device__ __forceinline__ FF ff_shfl_down(FF a, int o)
 {
     FF b;
@@ -888,26 +945,25 @@ __device__ __forceinline__ void publish_partial(double v, CGState *st, double *p
     }
 }
 
-// The sum of n block partials (doubles, or FP32 pairs), in thread 0 of every
-// block that calls it, in one order.
-template <int BS, bool PAIRS>
+// The sum of n block partials, in thread 0 of every block that calls it, in
+// one order.
+template <int BS>
+__device__ __forceinline__ FF sum_partials_ff(const double *partials, int n)
+{
+    __shared__ float2 smf[32];
+    FF acc = {0.f, 0.f};
+    for (int k = threadIdx.x; k < n; k += BS)
+        acc = ff_add(acc, ff_of(__ldcg(reinterpret_cast<const float2 *>(partials) + k)));
+    return block_sum_ff<BS>(acc, smf);
+}
+
+template <int BS>
 __device__ __forceinline__ double sum_partials(const double *partials, int n)
 {
-    if constexpr (PAIRS) {
-        __shared__ float2 smf[32];
-        FF acc = {0.f, 0.f};
-        for (int k = threadIdx.x; k < n; k += BS) {
-            const float2 p = __ldcg(reinterpret_cast<const float2 *>(partials) + k);
-            acc = ff_add(acc, FF{p.x, p.y});
-        }
-        const FF t = block_sum_ff<BS>(acc, smf);
-        return (double)t.hi + (double)t.lo;
-    } else {
-        __shared__ double sm[BS];
-        double acc = 0.0;
-        for (int k = threadIdx.x; k < n; k += BS) acc += __ldcg(partials + k);
-        return block_sum_smem<BS>(acc, sm);
-    }
+    __shared__ double sm[BS];
+    double acc = 0.0;
+    for (int k = threadIdx.x; k < n; k += BS) acc += __ldcg(partials + k);
+    return block_sum_smem<BS>(acc, sm);
 }
 
 template <int BS>
@@ -935,7 +991,7 @@ __device__ __forceinline__ bool grid_sum_ff(FF v, float2 *partials, unsigned *co
     }
     FF t = block_sum_ff<BS>(acc, smf);
     if (threadIdx.x == 0) {
-        total = (double)t.hi + (double)t.lo;
+        total = ff_double(t);
         *counter = 0u;
         return true;
     }

@@ -122,6 +122,31 @@ stg_status cuda_fail(cudaError_t e, const char *what);
 
 Geom make_geom(const int dims[4]);
 
+// The state's scalars as FP32 pairs for the mixed CG's kernels (before a copy
+// to the device, inner precision pd), and back (after one from it).
+inline float2 ff_split(double v)
+{
+    const float hi = (float)v;
+    return make_float2(hi, (float)(v - (double)hi));
+}
+inline void state_put(CGState *h, int pd)
+{
+    h->ff = pd != P64;
+    h->m2f = (float)h->m2;
+    h->trig2f = (float)h->trig2;
+    h->f_stop = ff_split(h->stop_r2);
+    h->f_delta = ff_split(h->delta_new);
+    h->f_delta_old = ff_split(h->delta_old);
+    h->f_rmax2 = ff_split(h->rmax2);
+}
+inline void state_got(CGState *h)
+{
+    if (!h->ff) return;
+    h->delta_new = (double)h->f_delta.x + (double)h->f_delta.y;
+    h->delta_old = (double)h->f_delta_old.x + (double)h->f_delta_old.y;
+    h->rmax2 = (double)h->f_rmax2.x + (double)h->f_rmax2.y;
+}
+
 // stg_cg_params defaults for inner iterations in `sloppy` (api.cu)
 void cg_params_for(int sloppy, stg_cg_params *p);
 
@@ -196,6 +221,7 @@ struct DslashArgs {
     const void *w;
     const void *v;
     double m2;
+    float m2f;          // m2 in FP32: a conversion per thread costs 16 cycles of the FP64 pipe a warp
     double *dot;
     CGState *state;
     double *partials;
