@@ -100,7 +100,9 @@ typedef struct stg_cg_params {
                           |r^y| < delta * max|r^y| since the last update       */
     long maxiter;      /* bound on the total iteration count (0 = 10 N_dim,
                           N_dim = 3 Vh as in Fig. 1)                           */
-    int check_every;   /* inner iterations between host checks (0 = auto)     */
+    int check_every;   /* inner iterations between host checks (0 = auto; small
+                          lattices with unitary links and timing = 0 are solved
+                          by one kernel, without host checks)                  */
     int timing;        /* 1: chunks rotate between timing the four kernels
                           of their first iteration with CUDA events recorded
                           inside the solver's graph, and timing whole chunks

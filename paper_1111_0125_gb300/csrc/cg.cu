@@ -666,6 +666,11 @@ stg_status cg_solve(stg_gauge *g, const double *src, double *x, double mass, dou
     Workspace *ws;
     STG_TRY(workspace_get(g, &ws));
     STG_TRY(prepare(g, ws, pd));
+    const int ctas = p->timing ? 0 : cluster_ctas(g, pd, 1, false);
+    if (ctas) {
+        const ClFields f = {ws->x64, ws->b64, ws->y, plain ? ws->r64 : ws->r, ws->d, ws->q, ws->tmp[pd]};
+        return cluster_solve(g, ws, ctas, 1, false, f, src, x, &mass, tol, p, pd, stats, s);
+    }
     const double m2 = mass * mass;
     const long maxiter = p->maxiter > 0 ? p->maxiter : 10L * 3L * geo.Vh;
     int chunk = p->check_every > 0 ? p->check_every : (geo.Vh >= (1 << 19) ? 16 : 32);

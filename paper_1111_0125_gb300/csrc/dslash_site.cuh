@@ -10,8 +10,8 @@
 
 namespace stg {
 
-// links and fields in floating point
-template <int P, int R>
+// links and fields in floating point; NC: no thread of the kernel writes `in`
+template <int P, int R, bool NC = true>
 __device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site_fp(const Geom &g, const Site &s,
                                                                     const char *const *lf,
                                                                     const char *const *lb, const void *in, int i)
@@ -30,10 +30,10 @@ __device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site_fp(const Geom &
         const T s2f = (R == 12) ? T(sf * LinkPost<P>::row2) : T(1);
         const T s2b = (R == 12) ? T(sb * LinkPost<P>::row2) : T(1);
         const Mat3<T> uf = LinkIO<P, R>::load(lf[mu], vh, i);
-        const Vec3<T> vf = FieldIO<P>::load_nc(in, vh, jf);
+        const Vec3<T> vf = FieldIO<P>::template load<NC>(in, vh, jf);
         mul_add<R == 12>(uf, vf, acc, s2f);
         const Mat3<T> ub = LinkIO<P, R>::load(lb[mu], vh, jb);
-        const Vec3<T> vb = FieldIO<P>::load_nc(in, vh, jb);
+        const Vec3<T> vb = FieldIO<P>::template load<NC>(in, vh, jb);
         adj_mul_sub(ub, vb, acc, s2b);
     }
     if (P == PX16) {
@@ -46,14 +46,14 @@ __device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site_fp(const Geom &
     return acc;
 }
 
-template <int P, int R>
+template <int P, int R, bool NC = true>
 __device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site(const Geom &g, const char *const *lf,
                                                                  const char *const *lb, int parity,
                                                                  const void *in, int i)
 {
     if constexpr (P == P64 && (R & kFixLinks) != 0) {
         constexpr int RC = R & ~kFixLinks;
-        return fix_site<RC>(g, parity, i, [&](const Site &s, int i, int mu, bool back) {
+        return fix_site<RC, NC>(g, parity, i, [&](const Site &s, int i, int mu, bool back) {
             int jf, jb;
             neighbours(g, s, i, mu, jf, jb);
             float sf = 1.f, sb = 1.f;
@@ -61,7 +61,7 @@ __device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site(const Geom &g, 
             return back ? FixHop{lb[mu], g.Vh, jb, in, g.Vh, jb, sb} : FixHop{lf[mu], g.Vh, i, in, g.Vh, jf, sf};
         });
     } else {
-        return dslash_site_fp<P, R>(g, site_of(g, i, parity), lf, lb, in, i);
+        return dslash_site_fp<P, R, NC>(g, site_of(g, i, parity), lf, lb, in, i);
     }
 }
 

@@ -89,7 +89,7 @@ __device__ __forceinline__ void fix_row2(FixLink &u, int s)
     }
 }
 
-template <int RC>
+template <int RC, bool PLAIN = false>
 __device__ __forceinline__ FixLink fix_link(const char *blk, int stride, int i, int s2)
 {
     const uint4 *p = reinterpret_cast<const uint4 *>(blk) + i;
@@ -97,7 +97,7 @@ __device__ __forceinline__ FixLink fix_link(const char *blk, int stride, int i, 
     constexpr int n = RC == 18 ? 9 : 6;
 #pragma unroll
     for (int k = 0; k < n; ++k) {
-        const uint4 a = ld_stream(p + (size_t)k * stride);
+        const uint4 a = ld_link<PLAIN>(p + (size_t)k * stride);
         u.h[k / 3][k % 3][0] = (int)a.x;
         u.l[k / 3][k % 3][0] = (int)a.y;
         u.h[k / 3][k % 3][1] = (int)a.z;
@@ -236,10 +236,10 @@ struct FixHop {
 // One hop in FP64 on the link's doubles (the recomputation): acc += U v, or
 // acc -= U^dag v for a backward hop.  Not inlined: it runs for exceptional
 // sites only, and inlined its registers made every site's path spill.
-template <int RC>
+template <int RC, bool NC>
 __device__ __noinline__ void fix_hop_f64(const FixHop t, bool back, Vec3<double> *acc)
 {
-    const Vec3<double> v = FieldIO<P64>::load_nc(t.f, t.fstride, t.fi);
+    const Vec3<double> v = FieldIO<P64>::load<NC>(t.f, t.fstride, t.fi);
     if (v.r[0] == 0.0 && v.i[0] == 0.0 && v.r[1] == 0.0 && v.i[1] == 0.0 && v.r[2] == 0.0 && v.i[2] == 0.0) return;
     const uint4 *p = reinterpret_cast<const uint4 *>(t.link) + t.li;
     Mat3<double> u;
@@ -258,7 +258,7 @@ __device__ __noinline__ void fix_hop_f64(const FixHop t, bool back, Vec3<double>
 }
 
 // D chi at site i; hop(s, i, mu, back) gives the eight hops' operands.
-template <int RC, class H>
+template <int RC, bool NC = true, class H>
 __device__ __forceinline__ Vec3<double> fix_site(const Geom &g, int parity, int i, const H &hop)
 {
     const Site s = site_of(g, i, parity);
@@ -269,12 +269,12 @@ __device__ __forceinline__ Vec3<double> fix_site(const Geom &g, int parity, int 
         {
             const FixHop t = hop(s, i, mu, false);
             const FixLink u = fix_link<RC>(t.link, t.lstride, t.li, t.s < 0.f ? -1 : 1);
-            fix_hop<false>(acc, u, FieldIO<P64>::load_nc(t.f, t.fstride, t.fi));
+            fix_hop<false>(acc, u, FieldIO<P64>::load<NC>(t.f, t.fstride, t.fi));
         }
         {
             const FixHop t = hop(s, i, mu, true);
             const FixLink u = fix_link<RC>(t.link, t.lstride, t.li, t.s < 0.f ? -1 : 1);
-            fix_hop<true>(acc, u, FieldIO<P64>::load_nc(t.f, t.fstride, t.fi));
+            fix_hop<true>(acc, u, FieldIO<P64>::load<NC>(t.f, t.fstride, t.fi));
         }
     }
     if (fix_ok(acc)) return fix_value(acc);
@@ -286,7 +286,7 @@ __device__ __forceinline__ Vec3<double> fix_site(const Geom &g, int parity, int 
 #pragma unroll
     for (int c = 0; c < 3; ++c) d.r[c] = d.i[c] = 0.0;
 #pragma unroll 1
-    for (int k = 0; k < 8; ++k) fix_hop_f64<RC>(hop(z, i, k >> 1, k & 1), k & 1, &d);
+    for (int k = 0; k < 8; ++k) fix_hop_f64<RC, NC>(hop(z, i, k >> 1, k & 1), k & 1, &d);
     return d;
 }
 

@@ -592,6 +592,8 @@ void workspace_free(Workspace *ws)
     if (!ws) return;
     batch_destroy(ws->batch);
     cudaFree(ws->mrhs_tmp);
+    cudaFree(ws->cl_dev);
+    if (ws->cl_host) cudaFreeHost(ws->cl_host);
     for (int k = 0; k < 3; ++k)
         if (ws->graph[k]) cudaGraphExecDestroy(ws->graph[k]);
     for (int k = 0; k < 5; ++k)

@@ -664,6 +664,12 @@ stg_status cg_solve_mrhs(stg_gauge *g, int n, const double *src, double *x, cons
         STG_TRY(batch_create(g, n, p, s, &b));
         ws->batch = b;
     }
+    const int ctas = getenv("STG_MRHS_SHAPE") ? 0 : cluster_ctas(g, p->sloppy, n, true);
+    if (ctas) {
+        const MrhsWs *m = b->m;
+        const ClFields f = {m->x64, m->b64, m->y, m->r, m->d, m->q, m->t};
+        return cluster_solve(g, ws, ctas, n, true, f, src, x, masses, tol, p, p->sloppy, stats, s);
+    }
     b->p = *p;
     b->s = s;
     b->launches = 0;

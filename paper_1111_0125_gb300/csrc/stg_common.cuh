@@ -453,9 +453,17 @@ __device__ __forceinline__ double2 ld_stream(const double2 *p)
     return v;
 }
 
+// PLAIN: an ordinary load, for records in shared memory or re-read from L1
+template <bool PLAIN, typename V> __device__ __forceinline__ V ld_link(const V *p)
+{
+    if constexpr (PLAIN) return *p;
+    else return ld_stream(p);
+}
+
 template <int P, int R> struct LinkIO;
 
 template <int R> struct LinkIO<P64, R> {
+    template <bool PLAIN = false>
     __device__ __forceinline__ static Mat3<double> load(const char *blk, int vh, int s)
     {
         const double2 *p = reinterpret_cast<const double2 *>(blk);
@@ -463,7 +471,7 @@ template <int R> struct LinkIO<P64, R> {
         constexpr int n = R == 18 ? 9 : 6;
 #pragma unroll
         for (int k = 0; k < n; ++k) {
-            double2 a = ld_stream(p + (size_t)k * vh + s);
+            double2 a = ld_link<PLAIN>(p + (size_t)k * vh + s);
             set_entry(u, k, a.x, a.y);
         }
         if (R == 12) reconstruct_row2(u, 1.0);
@@ -472,6 +480,7 @@ template <int R> struct LinkIO<P64, R> {
 };
 
 template <int R> struct LinkIO<P32, R> {
+    template <bool PLAIN = false>
     __device__ __forceinline__ static Mat3<float> load(const char *blk, int vh, int s)
     {
         const float4 *p = reinterpret_cast<const float4 *>(blk);
@@ -479,12 +488,12 @@ template <int R> struct LinkIO<P32, R> {
         constexpr int n4 = R == 18 ? 4 : 3;
 #pragma unroll
         for (int k = 0; k < n4; ++k) {
-            float4 a = ld_stream(p + (size_t)k * vh + s);
+            float4 a = ld_link<PLAIN>(p + (size_t)k * vh + s);
             set_entry(u, 2 * k, a.x, a.y);
             set_entry(u, 2 * k + 1, a.z, a.w);
         }
         if (R == 18) {
-            float2 b = ld_stream(reinterpret_cast<const float2 *>(p + (size_t)4 * vh) + s);
+            float2 b = ld_link<PLAIN>(reinterpret_cast<const float2 *>(p + (size_t)4 * vh) + s);
             set_entry(u, 8, b.x, b.y);
         } else {
             reconstruct_row2(u, 1.0f);
@@ -495,28 +504,29 @@ template <int R> struct LinkIO<P32, R> {
 
 // 16-bit float links (|U_ab| <= 1, no scale): entries as float pairs
 template <class C, int R> struct LinkIO16 {
+    template <bool PLAIN = false>
     __device__ __forceinline__ static Mat3<float> load(const char *blk, int vh, int s)
     {
         const uint4 *p = reinterpret_cast<const uint4 *>(blk);
         Mat3<float> u;
-        uint4 a = ld_stream(p + s);
+        uint4 a = ld_link<PLAIN>(p + s);
         float2 e0 = C::dec(a.x), e1 = C::dec(a.y), e2 = C::dec(a.z), e3 = C::dec(a.w);
         set_entry(u, 0, e0.x, e0.y);
         set_entry(u, 1, e1.x, e1.y);
         set_entry(u, 2, e2.x, e2.y);
         set_entry(u, 3, e3.x, e3.y);
         if (R == 18) {
-            uint4 b = ld_stream(p + (size_t)vh + s);
+            uint4 b = ld_link<PLAIN>(p + (size_t)vh + s);
             float2 f0 = C::dec(b.x), f1 = C::dec(b.y), f2 = C::dec(b.z), f3 = C::dec(b.w);
             set_entry(u, 4, f0.x, f0.y);
             set_entry(u, 5, f1.x, f1.y);
             set_entry(u, 6, f2.x, f2.y);
             set_entry(u, 7, f3.x, f3.y);
-            unsigned c = ld_stream(reinterpret_cast<const unsigned *>(p + (size_t)2 * vh) + s);
+            unsigned c = ld_link<PLAIN>(reinterpret_cast<const unsigned *>(p + (size_t)2 * vh) + s);
             float2 g = C::dec(c);
             set_entry(u, 8, g.x, g.y);
         } else {
-            uint2 b = ld_stream(reinterpret_cast<const uint2 *>(p + (size_t)vh) + s);
+            uint2 b = ld_link<PLAIN>(reinterpret_cast<const uint2 *>(p + (size_t)vh) + s);
             float2 f0 = C::dec(b.x), f1 = C::dec(b.y);
             set_entry(u, 4, f0.x, f0.y);
             set_entry(u, 5, f1.x, f1.y);
@@ -534,25 +544,26 @@ template <int R> struct LinkIO<PB16, R> : LinkIO16<CodecBF16, R> {};
 // accumulated sum by 1/32767 once per site (LinkPost).  Row 2 of a 12-real
 // link is s conj(r0 x r1) / 32767, which keeps it on the same 32767 scale.
 template <int R> struct LinkIO<PX16, R> {
+    template <bool PLAIN = false>
     __device__ __forceinline__ static Mat3<float> load(const char *blk, int vh, int s)
     {
         const uint4 *p = reinterpret_cast<const uint4 *>(blk);
         Mat3<float> u;
-        uint4 a = ld_stream(p + s);
+        uint4 a = ld_link<PLAIN>(p + s);
         set_entry(u, 0, fx_lo(a.x), fx_hi(a.x));
         set_entry(u, 1, fx_lo(a.y), fx_hi(a.y));
         set_entry(u, 2, fx_lo(a.z), fx_hi(a.z));
         set_entry(u, 3, fx_lo(a.w), fx_hi(a.w));
         if (R == 18) {
-            uint4 b = ld_stream(p + (size_t)vh + s);
+            uint4 b = ld_link<PLAIN>(p + (size_t)vh + s);
             set_entry(u, 4, fx_lo(b.x), fx_hi(b.x));
             set_entry(u, 5, fx_lo(b.y), fx_hi(b.y));
             set_entry(u, 6, fx_lo(b.z), fx_hi(b.z));
             set_entry(u, 7, fx_lo(b.w), fx_hi(b.w));
-            unsigned c = ld_stream(reinterpret_cast<const unsigned *>(p + (size_t)2 * vh) + s);
+            unsigned c = ld_link<PLAIN>(reinterpret_cast<const unsigned *>(p + (size_t)2 * vh) + s);
             set_entry(u, 8, fx_lo(c), fx_hi(c));
         } else {
-            uint2 b = ld_stream(reinterpret_cast<const uint2 *>(p + (size_t)vh) + s);
+            uint2 b = ld_link<PLAIN>(reinterpret_cast<const uint2 *>(p + (size_t)vh) + s);
             set_entry(u, 4, fx_lo(b.x), fx_hi(b.x));
             set_entry(u, 5, fx_lo(b.y), fx_hi(b.y));
             reconstruct_row2(u, 1.0f);

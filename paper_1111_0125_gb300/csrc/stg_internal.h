@@ -177,6 +177,7 @@ struct Workspace {
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // per-kernel events
     cudaEvent_t ev_chunk[2] = {nullptr, nullptr};                        // around plain chunks
     stg_batch *batch = nullptr;       // session cached for stg_cg_solve_mrhs
+    void *cl_dev = nullptr, *cl_host = nullptr;  // systems of cluster_solve (device, pinned)
     void *mrhs_tmp = nullptr;         // odd intermediates of stg_apply_A_mrhs
     size_t mrhs_tmp_bytes = 0;
 };
@@ -250,6 +251,14 @@ stg_status launch_accumulate_x(int pr, int vh, void *x64, const void *y, cudaStr
 stg_status launch_norm2(int prec, int vh, const void *v, CGState *st, double *partials, cudaStream_t s);
 stg_status launch_true_residual(stg_gauge *g, const void *x64, const void *b64, void *r64, void *t64,
                                 double m2, CGState *st, double *partials, cudaStream_t s);
+// whole solves of small lattices in one kernel (cg_cluster.cu)
+struct ClFields {
+    void *x64, *t64, *y, *r, *d, *q, *t;
+};
+int cluster_ctas(const stg_gauge *g, int pd, int nsys, bool batch);
+stg_status cluster_solve(stg_gauge *g, Workspace *ws, int ctas, int nsys, bool batch, const ClFields &buf, const double *src,
+                         double *x, const double *masses, double tol, const stg_cg_params *p, int pd,
+                         stg_cg_stats *stats, cudaStream_t s);
 stg_status pack_field(const Geom &g, int prec, const double *canon, void *out, cudaStream_t s);
 stg_status unpack_field(const Geom &g, int prec, const void *in, double *canon, cudaStream_t s);
 
