@@ -3,7 +3,7 @@
 //
 // An iteration of a small lattice is four kernels of 2 to 3 us whose work is
 // a fraction of that; the launches, the grid totals and, between chunks, the
-// host are the time.  Here the cluster's CTAs (16, or 8) split the sites, the
+// host are the time.  Here the cluster's CTAs (up to 16) split the sites, the
 // barriers between the phases are cluster barriers in hardware (no spinning,
 // all CTAs resident by construction), and the sums travel through distributed
 // shared memory: every CTA stores its partial into all CTAs' slots before a
