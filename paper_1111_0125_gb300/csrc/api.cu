@@ -221,6 +221,7 @@ stg_status stg_dslash(const stg_gauge *g, int out_parity, const void *in_dev, vo
     DeviceScope ds(g->device);
     DslashLaunch L = {};
     L.links = lf;
+    L.pdl = true;
     L.out_parity = out_parity;
     L.in = in_dev;
     L.out = out_dev;
@@ -243,6 +244,7 @@ static stg_status apply_A_impl(const stg_gauge *gc, double mass, const void *in_
     Workspace *ws = g->ws;
     DslashLaunch L = {};
     L.links = lf;
+    L.pdl = true;
     L.out_parity = 1;
     L.in = in_dev;
     L.out = tmp;

@@ -170,6 +170,8 @@ __global__ void __launch_bounds__(kBlock, kVecBlocksPerSM)
 k_cg_update_m(int vh, char *y, char *r, const char *d, const char *q, size_t sr, size_t sd,
               CGState *states, const double *dq, double *rr, const int *active, const int *nactive)
 {
+    pdl_wait();
+    pdl_trigger();
     if ((int)blockIdx.y >= *nactive) return;
     const int k = active[blockIdx.y];
     cg_update_body<PD, PR>(vh, y + k * sr, r + k * sr, d + k * sd, q + k * sd, states + k,
@@ -277,6 +279,8 @@ __global__ void __launch_bounds__(kBlock, kVecBlocksPerSM)
 k_xpay_m(int vh, const char *r, char *d, size_t sr, size_t sd, CGState *states, const double *rr,
          const int *active, const int *nactive)
 {
+    pdl_wait();
+    pdl_trigger();
     if ((int)blockIdx.y >= *nactive) return;
     const int k = active[blockIdx.y];
     xpay_body<PD, PR>(vh, r + k * sr, d + k * sd, states + k, rr + (size_t)k * gridDim.x);
@@ -460,8 +464,7 @@ stg_status launch_update_m(int pd, int vh, char *y, char *r, const char *d, cons
                            const int *nactive, int nslots, cudaStream_t s)
 {
     const dim3 grid(grid_vec(vh, nslots), nslots);
-    STG_DISPATCH_PD(pd, k_cg_update_m, vh, y, r, d, q, sr, sd, states, dq, rr, active, nactive);
-    STG_CUDA(cudaGetLastError());
+    STG_DISPATCH_PD_EX(pd, k_cg_update_m, true, vh, y, r, d, q, sr, sd, states, dq, rr, active, nactive);
     return STG_OK;
 }
 
@@ -469,8 +472,7 @@ stg_status launch_xpay_m(int pd, int vh, const char *r, char *d, size_t sr, size
                          const double *rr, const int *active, const int *nactive, int nslots, cudaStream_t s)
 {
     const dim3 grid(grid_vec(vh, nslots), nslots);
-    STG_DISPATCH_PD(pd, k_xpay_m, vh, r, d, sr, sd, states, rr, active, nactive);
-    STG_CUDA(cudaGetLastError());
+    STG_DISPATCH_PD_EX(pd, k_xpay_m, true, vh, r, d, sr, sd, states, rr, active, nactive);
     return STG_OK;
 }
 
@@ -510,6 +512,7 @@ stg_status launch_true_residual(stg_gauge *g, const void *x64, const void *b64, 
 {
     DslashLaunch L = {};
     L.links = &g->hi;
+    L.pdl = true;
     L.out_parity = 1;
     L.in = x64;
     L.out = t64;
@@ -635,6 +638,7 @@ static stg_status true_residual(stg_gauge *g, Workspace *ws, double m2, cudaStre
     const Geom &geo = g->geom;
     DslashLaunch L = {};
     L.links = &g->hi;
+    L.pdl = true;
     L.out_parity = 1;
     L.in = ws->x64;
     L.out = ws->tmp[P64];

@@ -332,6 +332,7 @@ static stg_status iteration_m(const stg_gauge *g, MrhsWs *m, const LinkField *lf
     a.active = m->active + 1;
     a.states = m->states;
     a.partials = reinterpret_cast<float2 *>(m->partials);
+    a.pdl = true;
     a.parity = 1;
     a.in = m->d;
     a.out = m->t;
@@ -753,6 +754,7 @@ stg_status stg_dslash_mrhs(const stg_gauge *g, int out_parity, int nrhs, const v
     int shape;
     STG_TRY(tune(g, lf, nrhs, in_dev, out_dev, fb, s, &shape));
     MrhsArgs a = {};
+    a.pdl = true;
     a.parity = out_parity;
     a.in = static_cast<const char *>(in_dev);
     a.out = static_cast<char *>(out_dev);
@@ -791,6 +793,7 @@ stg_status stg_apply_A_mrhs(const stg_gauge *gc, int nrhs, const double *masses,
     int shape;
     STG_TRY(tune(g, lf, nrhs, in_dev, ws->mrhs_tmp, fb, s, &shape));
     MrhsArgs a = {};
+    a.pdl = true;
     a.parity = 1;
     a.in = static_cast<const char *>(in_dev);
     a.out = static_cast<char *>(ws->mrhs_tmp);

@@ -40,6 +40,7 @@ struct MrhsArgs {
     CGState *states;       // per system (EPI_GATE, EPI_A_CG)
     float m2[kMaxRhs];     // EPI_A: m_k^2
     float2 *partials;      // EPI_A_CG: [nrhs][gridDim.x]
+    bool pdl;              // host: programmatic dependent launch (the kernels wait and trigger)
     int grid_cap;          // blocks launched at most (they stride over site tiles)
     int grid_limit;        // staged kernels: at most this many CTAs (0 = all resident;
                            // STG_MRHS_GRID, read per call, for tests)
@@ -75,6 +76,8 @@ __global__ void __launch_bounds__(kMrhsBlock) k_dslash_m(const MrhsArgs a)
 {
     constexpr int BS = kMrhsBlock;
     typedef typename Real<P>::T T;
+    pdl_wait();
+    pdl_trigger();
     const int vh = a.g.Vh;
     const int sub = threadIdx.x % TPS;
     const int nact = a.active ? *a.nactive : a.nrhs;
@@ -494,6 +497,9 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
             }
         }
     }
+    // the links are constant: the fills above overlap the previous kernel
+    pdl_wait();
+    pdl_trigger();
     if (EPI == EPI_GATE) commit_systems(a, nact);
     if (EPI == EPI_A_CG)
         for (int k = threadIdx.x; k < kMsWarps * kMaxRhs; k += kMsThreads)
@@ -806,10 +812,10 @@ void launch_ms_nb(int epi, const MrhsArgs &a, cudaStream_t s)
     if (a.grid_limit > 0 && a.grid_limit < cap) cap = a.grid_limit;
     const int grid = ntiles < cap ? ntiles : cap;
     switch (epi) {
-    case EPI_NONE: k_dslash_ms<P, NB, EPI_NONE, RI><<<grid, kMsThreads, smem, s>>>(a); break;
-    case EPI_A: k_dslash_ms<P, NB, EPI_A, RI><<<grid, kMsThreads, smem, s>>>(a); break;
-    case EPI_GATE: k_dslash_ms<P, NB, EPI_GATE, RI><<<grid, kMsThreads, smem, s>>>(a); break;
-    case EPI_A_CG: k_dslash_ms<P, NB, EPI_A_CG, RI><<<grid, kMsThreads, smem, s>>>(a); break;
+    case EPI_NONE: launch_k(k_dslash_ms<P, NB, EPI_NONE, RI>, grid, kMsThreads, smem, s, a.pdl, a); break;
+    case EPI_A: launch_k(k_dslash_ms<P, NB, EPI_A, RI>, grid, kMsThreads, smem, s, a.pdl, a); break;
+    case EPI_GATE: launch_k(k_dslash_ms<P, NB, EPI_GATE, RI>, grid, kMsThreads, smem, s, a.pdl, a); break;
+    case EPI_A_CG: launch_k(k_dslash_ms<P, NB, EPI_A_CG, RI>, grid, kMsThreads, smem, s, a.pdl, a); break;
     }
 }
 
@@ -857,10 +863,10 @@ void launch_m_pr(int shape, int epi, const MrhsArgs &a, cudaStream_t s)
         const long tiles_ = ((long)a.g.Vh * TPS_ + kMrhsBlock - 1) / kMrhsBlock;                      \
         const int grid = (int)(tiles_ < a.grid_cap ? tiles_ : a.grid_cap);                             \
         switch (epi) {                                                                                 \
-        case EPI_NONE: k_dslash_m<P, R, NB_, TPS_, EPI_NONE><<<grid, kMrhsBlock, 0, s>>>(a); break;    \
-        case EPI_A: k_dslash_m<P, R, NB_, TPS_, EPI_A><<<grid, kMrhsBlock, 0, s>>>(a); break;          \
-        case EPI_GATE: k_dslash_m<P, R, NB_, TPS_, EPI_GATE><<<grid, kMrhsBlock, 0, s>>>(a); break;    \
-        case EPI_A_CG: k_dslash_m<P, R, NB_, TPS_, EPI_A_CG><<<grid, kMrhsBlock, 0, s>>>(a); break;    \
+        case EPI_NONE: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_NONE>, grid, kMrhsBlock, 0, s, a.pdl, a); break;    \
+        case EPI_A: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_A>, grid, kMrhsBlock, 0, s, a.pdl, a); break;          \
+        case EPI_GATE: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_GATE>, grid, kMrhsBlock, 0, s, a.pdl, a); break;    \
+        case EPI_A_CG: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_A_CG>, grid, kMrhsBlock, 0, s, a.pdl, a); break;    \
         }                                                                                              \
     } while (0)
     switch (shape) {

@@ -70,6 +70,8 @@ __global__ void __launch_bounds__(kMspThreads, NB == 2 ? 4 : 3) k_dslash_msp(con
             }
         }
     }
+    pdl_wait();
+    pdl_trigger();
     if (EPI == EPI_GATE) commit_systems(a, nact);
     if (EPI == EPI_A_CG)
         for (int k = threadIdx.x; k < kMspWarps * kMaxRhs; k += kMspThreads)
@@ -246,10 +248,10 @@ void launch_msp_nb(int epi, const MrhsArgs &a, cudaStream_t s)
     if (a.grid_limit > 0 && a.grid_limit < cap) cap = a.grid_limit;
     const int grid = ntiles < cap ? ntiles : cap;
     switch (epi) {
-    case EPI_NONE: k_dslash_msp<NB, EPI_NONE><<<grid, kMspThreads, smem, s>>>(a); break;
-    case EPI_A: k_dslash_msp<NB, EPI_A><<<grid, kMspThreads, smem, s>>>(a); break;
-    case EPI_GATE: k_dslash_msp<NB, EPI_GATE><<<grid, kMspThreads, smem, s>>>(a); break;
-    case EPI_A_CG: k_dslash_msp<NB, EPI_A_CG><<<grid, kMspThreads, smem, s>>>(a); break;
+    case EPI_NONE: launch_k(k_dslash_msp<NB, EPI_NONE>, grid, kMspThreads, smem, s, a.pdl, a); break;
+    case EPI_A: launch_k(k_dslash_msp<NB, EPI_A>, grid, kMspThreads, smem, s, a.pdl, a); break;
+    case EPI_GATE: launch_k(k_dslash_msp<NB, EPI_GATE>, grid, kMspThreads, smem, s, a.pdl, a); break;
+    case EPI_A_CG: launch_k(k_dslash_msp<NB, EPI_A_CG>, grid, kMspThreads, smem, s, a.pdl, a); break;
     }
 }
 

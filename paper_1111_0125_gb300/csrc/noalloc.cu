@@ -119,6 +119,7 @@ extern "C" stg_status stg_apply_A_dot_noalloc(const stg_gauge *g, double mass, c
         void *tmp = base + off_tmp;
         DslashLaunch L = {};
         L.links = lf;
+        L.pdl = true;
         L.out_parity = 1;
         L.in = in_dev;
         L.out = tmp;

@@ -201,7 +201,9 @@ struct DslashLaunch {
     CGState *state;  // EPI_A_CG, EPI_GATE
     double *partials;
     unsigned *counter;
-    bool pdl;        // programmatic dependent launch (inside the CG graph)
+    bool pdl;        // programmatic dependent launch: the kernel's blocks are
+                     // placed while the previous kernel of the stream drains
+                     // and wait for its end before they touch a field
 };
 
 stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &a, cudaStream_t s);

@@ -20,3 +20,52 @@ def test_one_site_kernel_runs(dims, prec, recon):
             group = torch.empty_like(f)
             stg.stg_dslash_group([g.handle], [parity], [f], [group], prec)
             assert torch.equal(g.dslash(f, parity, prec), group)
+
+
+@pytest.mark.parametrize("prec,recon", [(stg.STG_FP64, 18), (stg.STG_FP32, 12), (stg.STG_FP16, 12)])
+def test_early_placed_blocks_wait_for_the_input(prec, recon):
+    """The operators' kernels may be placed while their predecessor runs; the
+    input's producer is a copy, a memset, another library's kernel or another
+    stream's, eagerly and in a captured graph, and the output never changes."""
+    dims, mass = (16, 16, 16, 16), 0.1
+    with stg.Gauge(dims, gen.gauge_field(dims, "exp", seed=1, eps=0.5), sloppy=prec, recon=recon) as g:
+        x = g.pack(torch.from_numpy(gen.source(dims, seed=2)).cuda(), prec)
+        f, out, dot = torch.empty_like(x), torch.empty_like(x), torch.empty(1, dtype=torch.float64, device="cuda")
+        side = torch.cuda.Stream()
+
+        def call():
+            stg.stg_apply_A_dot(g.handle, mass, f, out, dot, prec)
+
+        def produce(kind):
+            f.zero_()
+            if kind == 0:
+                f.copy_(x)
+            elif kind == 1:
+                f.add_(x)
+            else:
+                cur = torch.cuda.current_stream()
+                side.wait_stream(cur)
+                with torch.cuda.stream(side):
+                    f.copy_(x)
+                cur.wait_stream(side)
+
+        f.copy_(x)
+        call()
+        want, want_dot = out.clone(), dot.clone()
+        for k in range(30):
+            produce(k % 3)
+            call()
+            got = out.clone()
+            assert torch.equal(got, want) and torch.equal(dot, want_dot)
+        stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+        stream.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(stream), torch.cuda.graph(graph, stream=stream):
+            call()
+            for kind in range(3):
+                produce(kind)
+                call()
+        for _ in range(5):
+            out.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(out, want) and torch.equal(dot, want_dot)
