@@ -30,14 +30,33 @@ namespace stg {
 // 24^3x48, A with its dot, 18-real / 12-real: 145 / 208 us; three blocks (80
 // registers, 150-550 bytes spilled) 146 / 224 us; one block (200 registers)
 // 193 / 270 us.
-constexpr int min_blocks(int p, int r) { return p == P64 && (r & kFixLinks) ? 2 : 1; }
+constexpr int min_blocks(int p, int r, int bs) { return (p == P64 && (r & kFixLinks) ? 2 : 1) * (kBlock / bs); }
+
+// Threads per block.  Blocks of 128 put a small lattice on twice the SMs and
+// even out the last wave of a large one; between, blocks of 256 leave fewer
+// partials and share more neighbours in L1.  Measured (us, 256 against 128
+// threads): A with its dot on Vh 2048: FP32/12 6.1 / 5.4, FP64/18 18.8 / 14.7;
+// 10368: 6.1 / 5.5, 18.8 / 14.7; 20736: 6.5 / 6.5; 49152: 9.3 / 10.0; 65536 BF16/18
+// 9.6 / 10.9; half-pass on 331776: FP32/12 20.5 / 20.0, FP32/18 30.5 / 29.4, BF16/18
+// 17.6 / 16.7, FP64/18 63.9 / 62.7, but FP64/12 97.6 / 103.8.  Sums keep 256 on
+// large lattices: one partial per 256 sites is what their scratch holds.
+constexpr int kSmallBlock = 128;
+constexpr int kSmallMax = 16384;  // ceil(Vh / 128) partials fit ceil(Vh / 256) + 64 up to here
+
+int dslash_blocks(int vh, int epi, bool limbs12)
+{
+    const bool sums = epi == EPI_A_DOT || epi == EPI_A_CG || epi == EPI_RES;
+    const bool fine = vh <= kSmallMax || (!sums && !limbs12 && vh >= 200000);
+    const int bs = fine ? kSmallBlock : kBlock;
+    return (vh + bs - 1) / bs;
+}
 
 template <typename T> __device__ __forceinline__ T pick_m2(double d, float f);
 template <> __device__ __forceinline__ double pick_m2<double>(double d, float) { return d; }
 template <> __device__ __forceinline__ float pick_m2<float>(double, float f) { return f; }
 
-template <int P, int R, int EPI>
-__global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const DslashArgs a)
+template <int P, int R, int EPI, int BS>
+__global__ void __launch_bounds__(BS, min_blocks(P, R, BS)) k_dslash(const DslashArgs a)
 {
     typedef typename Real<P>::T T;
     pdl_wait();
@@ -46,7 +65,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const Dslas
         if (a.state->flag != FLAG_RUN) return;  // uniform over the grid
         if (EPI == EPI_GATE && blockIdx.x == 0 && threadIdx.x == 0) cg_commit(a.state);
     }
-    const int i = blockIdx.x * kBlock + threadIdx.x;
+    const int i = blockIdx.x * BS + threadIdx.x;
     const int vh = a.g.Vh;
     T dot = T(0);
     if (i < vh) {
@@ -82,27 +101,35 @@ __global__ void __launch_bounds__(kBlock, min_blocks(P, R)) k_dslash(const Dslas
         }
     }
     if constexpr (EPI == EPI_A_CG) {
-        if constexpr (P == P64) publish_partial<kBlock>(double(dot), a.state, a.partials);
-        else publish_partial<kBlock>(FF{float(dot), 0.f}, a.state, a.partials);
+        if constexpr (P == P64) publish_partial<BS>(double(dot), a.state, a.partials);
+        else publish_partial<BS>(FF{float(dot), 0.f}, a.state, a.partials);
     } else if constexpr (EPI == EPI_A_DOT || EPI == EPI_RES) {
         double total;
         bool last;
-        if constexpr (P == P64) last = grid_sum<kBlock>(double(dot), a.partials, a.counter, total);
-        else last = grid_sum_ff<kBlock>(FF{float(dot), 0.f}, reinterpret_cast<float2 *>(a.partials), a.counter, total);
+        if constexpr (P == P64) last = grid_sum<BS>(double(dot), a.partials, a.counter, total);
+        else last = grid_sum_ff<BS>(FF{float(dot), 0.f}, reinterpret_cast<float2 *>(a.partials), a.counter, total);
         if (last) *a.dot = total;
     }
 }
 
+template <int P, int R, int EPI>
+static void launch_bs(const DslashArgs &a, cudaStream_t s, bool pdl)
+{
+    const int vh = a.g.Vh, grid = dslash_blocks(vh, EPI, P == P64 && R == (12 | kFixLinks));
+    if (grid == (vh + kBlock - 1) / kBlock) launch_k(k_dslash<P, R, EPI, kBlock>, grid, kBlock, 0, s, pdl, a);
+    else launch_k(k_dslash<P, R, EPI, kSmallBlock>, grid, kSmallBlock, 0, s, pdl, a);
+}
+
 template <int P, int R>
-static void launch_pr(int epi, const DslashArgs &a, int grid, cudaStream_t s, bool pdl)
+static void launch_pr(int epi, const DslashArgs &a, cudaStream_t s, bool pdl)
 {
     switch (epi) {
-    case EPI_NONE: launch_k(k_dslash<P, R, EPI_NONE>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A: launch_k(k_dslash<P, R, EPI_A>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A_DOT: launch_k(k_dslash<P, R, EPI_A_DOT>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A_CG: launch_k(k_dslash<P, R, EPI_A_CG>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_RES: launch_k(k_dslash<P, R, EPI_RES>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_GATE: launch_k(k_dslash<P, R, EPI_GATE>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_NONE: launch_bs<P, R, EPI_NONE>(a, s, pdl); break;
+    case EPI_A: launch_bs<P, R, EPI_A>(a, s, pdl); break;
+    case EPI_A_DOT: launch_bs<P, R, EPI_A_DOT>(a, s, pdl); break;
+    case EPI_A_CG: launch_bs<P, R, EPI_A_CG>(a, s, pdl); break;
+    case EPI_RES: launch_bs<P, R, EPI_RES>(a, s, pdl); break;
+    case EPI_GATE: launch_bs<P, R, EPI_GATE>(a, s, pdl); break;
     }
 }
 
@@ -128,7 +155,6 @@ stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &L
     a.state = L.state;
     a.partials = L.partials;
     a.counter = L.counter;
-    const int grid = (g.Vh + kBlock - 1) / kBlock;
     const int recon = L.links->recon;
     if (prec != L.links->prec) {
         set_error("dslash: link precision does not match the field precision");
@@ -139,25 +165,25 @@ stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &L
         return STG_OK;
     }
     if (prec == P64 && L.links->fix) {  // links as limbs: the integer form
-        if (recon == 18) launch_pr<P64, 18 | kFixLinks>(epi, a, grid, s, L.pdl);
-        else launch_pr<P64, 12 | kFixLinks>(epi, a, grid, s, L.pdl);
+        if (recon == 18) launch_pr<P64, 18 | kFixLinks>(epi, a, s, L.pdl);
+        else launch_pr<P64, 12 | kFixLinks>(epi, a, s, L.pdl);
     } else if (prec == P64) {
-        if (recon == 18) launch_pr<P64, 18>(epi, a, grid, s, L.pdl);
-        else launch_pr<P64, 12>(epi, a, grid, s, L.pdl);
+        if (recon == 18) launch_pr<P64, 18>(epi, a, s, L.pdl);
+        else launch_pr<P64, 12>(epi, a, s, L.pdl);
     } else if (prec == P32) {
-        if (recon == 18) launch_pr<P32, 18>(epi, a, grid, s, L.pdl);
-        else launch_pr<P32, 12>(epi, a, grid, s, L.pdl);
+        if (recon == 18) launch_pr<P32, 18>(epi, a, s, L.pdl);
+        else launch_pr<P32, 12>(epi, a, s, L.pdl);
     } else {
         if (prec == PB16) {
-            if (recon == 18) launch_pr<PB16, 18>(epi, a, grid, s, L.pdl);
-            else launch_pr<PB16, 12>(epi, a, grid, s, L.pdl);
+            if (recon == 18) launch_pr<PB16, 18>(epi, a, s, L.pdl);
+            else launch_pr<PB16, 12>(epi, a, s, L.pdl);
         } else if (prec == PX16) {
-            if (recon == 18) launch_pr<PX16, 18>(epi, a, grid, s, L.pdl);
-            else launch_pr<PX16, 12>(epi, a, grid, s, L.pdl);
+            if (recon == 18) launch_pr<PX16, 18>(epi, a, s, L.pdl);
+            else launch_pr<PX16, 12>(epi, a, s, L.pdl);
         } else if (recon == 18) {
-            launch_pr<P16, 18>(epi, a, grid, s, L.pdl);
+            launch_pr<P16, 18>(epi, a, s, L.pdl);
         } else {
-            launch_pr<P16, 12>(epi, a, grid, s, L.pdl);
+            launch_pr<P16, 12>(epi, a, s, L.pdl);
         }
     }
     STG_CUDA(cudaGetLastError());

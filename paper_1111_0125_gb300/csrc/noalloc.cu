@@ -82,11 +82,10 @@ extern "C" stg_status stg_apply_A_dot_noalloc(const stg_gauge *g, double mass, c
         return STG_ERR_UNSUPPORTED;
     }
     const Geom &geo = g->geom;
-    // every EPI_A_DOT launch writes one partial (8 bytes) per thread block
-    // and uses at most ceil(Vh / kBlock) blocks: one site per thread in
-    // k_dslash, two in k_dslash_fx2, and at most one block per 1024-site
-    // tile in the staged FX16 kernel
-    const size_t n_blocks = (size_t)(geo.Vh + kBlock - 1) / kBlock;
+    // every EPI_A_DOT launch writes one partial (8 bytes) per thread block:
+    // those of k_dslash, and fewer in k_dslash_fx2 (two sites per thread) and
+    // the staged 16-bit kernel (at most one block per 1024-site tile)
+    const size_t n_blocks = (size_t)dslash_blocks(geo.Vh, EPI_A_DOT, false);
     const size_t off_partials = 256;  // the counter lives in the first 256 bytes
     const size_t off_tmp = off_partials + round256(n_blocks * sizeof(double));
     const size_t need = off_tmp + round256((size_t)geo.Vh * field_site_bytes(prec));

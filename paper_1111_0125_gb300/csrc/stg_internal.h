@@ -207,6 +207,9 @@ struct DslashLaunch {
 };
 
 stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &a, cudaStream_t s);
+// thread blocks (and block partials) of the one-site kernel; limbs12: FP64 / 12-
+// real limb links
+int dslash_blocks(int vh, int epi, bool limbs12);
 
 // kernel arguments of every Dslash variant
 struct DslashArgs {
