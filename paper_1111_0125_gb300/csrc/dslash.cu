@@ -59,6 +59,7 @@ template <int P, int R, int EPI, int BS>
 __global__ void __launch_bounds__(BS, min_blocks(P, R, BS)) k_dslash(const DslashArgs a)
 {
     typedef typename Real<P>::T T;
+    constexpr int kUnroll = P == P64 && R == (12 | kFixLinks) && BS == kSmallBlock ? 2 : 4;  // see fix_site
     pdl_wait();
     pdl_trigger();
     if (EPI == EPI_A_CG || EPI == EPI_GATE) {
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(BS, min_blocks(P, R, BS)) k_dslash(const Dslas
     const int vh = a.g.Vh;
     T dot = T(0);
     if (i < vh) {
-        const Vec3<T> acc = dslash_site<P, R>(a.g, a.lf, a.lb, a.parity, a.in, i);
+        const Vec3<T> acc = dslash_site<P, R, true, kUnroll>(a.g, a.lf, a.lb, a.parity, a.in, i);
         if (EPI == EPI_NONE || EPI == EPI_GATE) {
             FieldIO<P>::store(a.out, vh, i, acc);
         } else if (EPI == EPI_RES) {

@@ -46,14 +46,14 @@ __device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site_fp(const Geom &
     return acc;
 }
 
-template <int P, int R, bool NC = true>
+template <int P, int R, bool NC = true, int U = 4>
 __device__ __forceinline__ Vec3<typename Real<P>::T> dslash_site(const Geom &g, const char *const *lf,
                                                                  const char *const *lb, int parity,
                                                                  const void *in, int i)
 {
     if constexpr (P == P64 && (R & kFixLinks) != 0) {
         constexpr int RC = R & ~kFixLinks;
-        return fix_site<RC, NC>(g, parity, i, [&](const Site &s, int i, int mu, bool back) {
+        return fix_site<RC, NC, U>(g, parity, i, [&](const Site &s, int i, int mu, bool back) {
             int jf, jb;
             neighbours(g, s, i, mu, jf, jb);
             float sf = 1.f, sb = 1.f;

@@ -257,14 +257,17 @@ __device__ __noinline__ void fix_hop_f64(const FixHop t, bool back, Vec3<double>
     *acc = d;
 }
 
-// D chi at site i; hop(s, i, mu, back) gives the eight hops' operands.
-template <int RC, bool NC = true, class H>
+// D chi at site i; hop(s, i, mu, back) gives the eight hops' operands.  U: the
+// directions unrolled; all four, but two in the 12-real kernels of small
+// lattices, whose code (64 KB unrolled) would come from L2 once per launch when
+// two of them alternate: A on 8^4 30.2 -> 22.3 us.  Elsewhere two cost 4-8%.
+template <int RC, bool NC = true, int U = 4, class H>
 __device__ __forceinline__ Vec3<double> fix_site(const Geom &g, int parity, int i, const H &hop)
 {
     const Site s = site_of(g, i, parity);
     FixAcc acc;
     fix_init(acc);
-#pragma unroll
+#pragma unroll U
     for (int mu = 0; mu < 4; ++mu) {
         {
             const FixHop t = hop(s, i, mu, false);

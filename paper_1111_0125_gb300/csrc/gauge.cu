@@ -207,13 +207,11 @@ stg_status links_check(const double2 *ucan, long n, int *bad, cudaStream_t s)
     return STG_OK;
 }
 
-stg_status links_fix(const Geom &g, LinkField *lf, cudaStream_t s)
+stg_status links_fix(LinkField *lf, cudaStream_t s)
 {
-    // every block holds Vh records in planes, all of them (re, im) pairs
-    const long n = (long)g.Vh * (link_bytes(P64, lf->recon) / 16);
-    for (int b = 0; b < 8; ++b)
-        k_fix_links<<<(int)((n + 255) / 256), 256, 0, s>>>(
-            n, reinterpret_cast<double2 *>(lf->base + (size_t)b * lf->blk_bytes));
+    // the eight blocks hold (re, im) pairs only; the padding between them goes along
+    const long n = (long)(8 * lf->blk_bytes / 16);
+    k_fix_links<<<(int)((n + 255) / 256), 256, 0, s>>>(n, reinterpret_cast<double2 *>(lf->base));
     STG_CUDA(cudaGetLastError());
     lf->fix = true;
     return STG_OK;
@@ -504,7 +502,7 @@ stg_status gauge_create(const int dims[4], const double *links_host, int sloppy,
     e = cudaStreamSynchronize(s);
     if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
     if (st == STG_OK && !bad) {
-        st = links_fix(g->geom, &g->hi, s);
+        st = links_fix(&g->hi, s);
         e = cudaStreamSynchronize(s);
         if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
     }

@@ -1168,7 +1168,7 @@ stg_status stg_slabs_create(const int dims[4], const double *links_host, int nsl
     cudaFree(ucan);
     if (st == STG_OK && !bad) {
         for (int r = 0; r < P && st == STG_OK; ++r)
-            st = links_fix(h->g, prec != STG_FP64 ? &h->links64[r] : &h->links[r], s);
+            st = links_fix(prec != STG_FP64 ? &h->links64[r] : &h->links[r], s);
         h->fix = true;
     }
     if (st == STG_OK) st = sl_alloc((void **)&h->ghost, (size_t)P * 2 * h->ghost_bytes);

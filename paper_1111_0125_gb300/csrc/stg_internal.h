@@ -156,7 +156,7 @@ const LinkField *links_for(const stg_gauge *g, int prec);
 // of n canonical links is not unitary; links_fix converts a packed FP64 field
 // in place
 stg_status links_check(const double2 *ucan, long n, int *bad, cudaStream_t s);
-stg_status links_fix(const Geom &g, LinkField *lf, cudaStream_t s);
+stg_status links_fix(LinkField *lf, cudaStream_t s);
 
 // Reduction scratch: partial sums (one double per block) and the state.
 struct Workspace {
