@@ -19,6 +19,8 @@
 
 #include <stdlib.h>
 
+#include <type_traits>
+
 #include "stg_internal.h"
 
 namespace stg {
@@ -568,11 +570,13 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
             __syncthreads();
         }
 
-        for (int k0 = 0; k0 < per; k0 += NB) {
-            int rid[NB];
-            bool run[NB];
+        // NQ list slots of this group from slot k0 on
+        const auto pass = [&](auto nq, int k0) {
+            constexpr int NQ = decltype(nq)::value;
+            int rid[NQ];
+            bool run[NQ];
 #pragma unroll
-            for (int q = 0; q < NB; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 const int kk = grp + kMsGroups * (k0 + q);
                 run[q] = kk < nact;
                 rid[q] = run[q] ? (a.active ? a.active[kk] : kk) : 0;
@@ -584,35 +588,35 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
                 // system after the eight mat-vecs: start those reads into L1
                 // now (measured: A of 16 systems at 24^3x48 244 -> 228 us)
 #pragma unroll
-                for (int q = 0; q < NB; ++q) {
+                for (int q = 0; q < NQ; ++q) {
                     const char *w = a.w + rid[q] * a.fstride;
                     prefetch_l1(w + (size_t)iv * 16);
                     if (P == P32) prefetch_l1(w + (size_t)vh * 16 + (size_t)iv * 8);
                 }
             }
-            Vec3<T> acc[NB];
-            // no branches in the hot loop: a slot that is not running reads
-            // system rid = 0 (valid memory) and its result is dropped below
+            Vec3<T> acc[NQ];
+            // no branches in the hot loop: a slot that is not running reads its
+            // system's fields (or those of system 0) and its result is dropped
             if constexpr (P == PX16 && !RI) {
                 // systems 2p and 2p + 1 share float2 accumulators: the decode
                 // of the 16-bit fields leaves the FMA pipe the busier one
-                float2 ar[NB / 2][3], ai[NB / 2][3];
+                float2 ar[NQ / 2][3], ai[NQ / 2][3];
 #pragma unroll
-                for (int p2 = 0; p2 < NB / 2; ++p2)
+                for (int p2 = 0; p2 < NQ / 2; ++p2)
 #pragma unroll
                     for (int c = 0; c < 3; ++c) ar[p2][c] = ai[p2][c] = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int mu = 0; mu < 4; ++mu) {
                     // both neighbours' fields of every system in flight at once
-                    Vec3<T> vf[NB], vb[NB];
+                    Vec3<T> vf[NQ], vb[NQ];
 #pragma unroll
-                    for (int q = 0; q < NB; ++q) {
+                    for (int q = 0; q < NQ; ++q) {
                         vf[q] = FieldIO<P>::load_nc(a.in + rid[q] * a.fstride, vh, jf[mu]);
                         vb[q] = FieldIO<P>::load_nc(a.in + rid[q] * a.fstride, vh, jb[mu]);
                     }
                     const Mat3<T> uf = MsLink<P>::load(sb + (size_t)(2 * mu) * LB, site, s2f[mu]);
 #pragma unroll
-                    for (int p2 = 0; p2 < NB / 2; ++p2) {
+                    for (int p2 = 0; p2 < NQ / 2; ++p2) {
                         float2 vr[3], vi[3];
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
@@ -623,7 +627,7 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
                     }
                     const Mat3<T> ub = MsLink<P>::load(sb + (size_t)(2 * mu + 1) * LB, site, s2b[mu]);
 #pragma unroll
-                    for (int p2 = 0; p2 < NB / 2; ++p2) {
+                    for (int p2 = 0; p2 < NQ / 2; ++p2) {
                         float2 vr[3], vi[3];
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
@@ -634,7 +638,7 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
                     }
                 }
 #pragma unroll
-                for (int p2 = 0; p2 < NB / 2; ++p2)
+                for (int p2 = 0; p2 < NQ / 2; ++p2)
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         acc[2 * p2].r[c] = ar[p2][c].x;
@@ -643,27 +647,27 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
                         acc[2 * p2 + 1].i[c] = ai[p2][c].y;
                     }
             } else if constexpr (RI) {
-                float2 A[NB][3], B[NB][3];
+                float2 A[NQ][3], B[NQ][3];
 #pragma unroll
-                for (int q = 0; q < NB; ++q)
+                for (int q = 0; q < NQ; ++q)
 #pragma unroll
                     for (int c = 0; c < 3; ++c) A[q][c] = B[q][c] = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int mu = 0; mu < 4; ++mu) {
                     // one direction's fields at a time (the accumulators
                     // take twice the registers of the scalar form)
-                    float2 v[NB][3];
+                    float2 v[NQ][3];
 #pragma unroll
-                    for (int q = 0; q < NB; ++q) {
+                    for (int q = 0; q < NQ; ++q) {
                         if constexpr (P == P32) load_ri(a.in + rid[q] * a.fstride, vh, jf[mu], v[q]);
                         else load_ri_fx(a.in + rid[q] * a.fstride, jf[mu], v[q]);
                     }
                     const Mat3<T> uf = (P == P32)
                         ? ms_link_ri(sb + (size_t)(2 * mu) * LB, row2s4 + 2 * mu * kMTile, row2s2 + 2 * mu * kMTile, site)
                         : ms_link_fx(lkx4 + 4 * (2 * mu) * kMTile, lkx2 + (2 * mu) * kMTile, site);
-                    mul_add_ri<NB>(uf, v, A, B);
+                    mul_add_ri<NQ>(uf, v, A, B);
 #pragma unroll
-                    for (int q = 0; q < NB; ++q) {
+                    for (int q = 0; q < NQ; ++q) {
                         if constexpr (P == P32) load_ri(a.in + rid[q] * a.fstride, vh, jb[mu], v[q]);
                         else load_ri_fx(a.in + rid[q] * a.fstride, jb[mu], v[q]);
                     }
@@ -671,10 +675,10 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
                         ? ms_link_ri(sb + (size_t)(2 * mu + 1) * LB, row2s4 + (2 * mu + 1) * kMTile,
                                      row2s2 + (2 * mu + 1) * kMTile, site)
                         : ms_link_fx(lkx4 + 4 * (2 * mu + 1) * kMTile, lkx2 + (2 * mu + 1) * kMTile, site);
-                    adj_mul_sub_ri<NB>(ub, v, A, B);
+                    adj_mul_sub_ri<NQ>(ub, v, A, B);
                 }
 #pragma unroll
-                for (int q = 0; q < NB; ++q)
+                for (int q = 0; q < NQ; ++q)
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         acc[q].r[c] = A[q][c].x - B[q][c].y;
@@ -684,28 +688,28 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
                 // FP32: scalar FMAs (packing the fields of two systems would
                 // cost more moves than it saves; RI avoids the moves)
 #pragma unroll
-                for (int q = 0; q < NB; ++q)
+                for (int q = 0; q < NQ; ++q)
 #pragma unroll
                     for (int c = 0; c < 3; ++c) acc[q].r[c] = acc[q].i[c] = T(0);
 #pragma unroll
                 for (int mu = 0; mu < 4; ++mu) {
-                    Vec3<T> vf[NB], vb[NB];
+                    Vec3<T> vf[NQ], vb[NQ];
 #pragma unroll
-                    for (int q = 0; q < NB; ++q) {
+                    for (int q = 0; q < NQ; ++q) {
                         vf[q] = FieldIO<P>::load_nc(a.in + rid[q] * a.fstride, vh, jf[mu]);
                         vb[q] = FieldIO<P>::load_nc(a.in + rid[q] * a.fstride, vh, jb[mu]);
                     }
                     const Mat3<T> uf = MsLink<P>::load(sb + (size_t)(2 * mu) * LB, site, T(1));
 #pragma unroll
-                    for (int q = 0; q < NB; ++q) mul_add(uf, vf[q], acc[q], s2f[mu]);
+                    for (int q = 0; q < NQ; ++q) mul_add(uf, vf[q], acc[q], s2f[mu]);
                     const Mat3<T> ub = MsLink<P>::load(sb + (size_t)(2 * mu + 1) * LB, site, T(1));
 #pragma unroll
-                    for (int q = 0; q < NB; ++q) adj_mul_sub(ub, vb[q], acc[q], s2b[mu]);
+                    for (int q = 0; q < NQ; ++q) adj_mul_sub(ub, vb[q], acc[q], s2b[mu]);
                 }
             }
-            FF dot[NB];
+            FF dot[NQ];
 #pragma unroll
-            for (int q = 0; q < NB; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 dot[q].hi = dot[q].lo = 0.f;
                 if (!ok || !run[q]) continue;
                 if (P == PX16 && !RI) {  // RI: the links carry 1/32767 already
@@ -737,13 +741,26 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
             if (EPI == EPI_A_CG) {
                 // a warp's 32 lanes are sites of one group: the same systems
 #pragma unroll
-                for (int q = 0; q < NB; ++q) {
+                for (int q = 0; q < NQ; ++q) {
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) dot[q] = ff_add(dot[q], ff_shfl_down(dot[q], o));
                     const int kk = grp + kMsGroups * (k0 + q);
                     if (lane == 0 && kk < nact) sysw[warp][kk] = ff_add(sysw[warp][kk], dot[q]);
                 }
             }
+        };
+        if constexpr (RI && NB == 2) {
+            // a group's odd last slot in a pass of its own, and nothing for a
+            // group without one: padded to NB, five systems cost as much as
+            // eight and two as much as four (A on 24^3x48: n = 2 113 -> 70 us, n = 5
+            // 129 -> 118, 12^3x24 n = 5 12.4 -> 11.2).  With NB = 4 the extra
+            // bodies cost its full passes 7%.
+            const int mine = (nact - grp + kMsGroups - 1) / kMsGroups;
+            int k0 = 0;
+            for (; k0 + 2 <= mine; k0 += 2) pass(std::integral_constant<int, 2>{}, k0);
+            if (k0 < mine) pass(std::integral_constant<int, 1>{}, k0);
+        } else {
+            for (int k0 = 0; k0 < per; k0 += NB) pass(std::integral_constant<int, NB>{}, k0);
         }
         // release the stage: the last warp to finish refills it
         __syncwarp();

@@ -69,3 +69,24 @@ def test_early_placed_blocks_wait_for_the_input(prec, recon):
             graph.replay()
             torch.cuda.synchronize()
             assert torch.equal(out, want) and torch.equal(dot, want_dot)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 7])
+@pytest.mark.parametrize("prec,tol", [(stg.STG_FP32, 1e-6), (stg.STG_FX16, 1e-4)])
+def test_batches_with_empty_and_odd_groups(n, prec, tol, monkeypatch):
+    """The staged multi-system kernel's four site groups share the systems; at
+    these sizes some have none or a single last one.  Against the single-system
+    A (each within the precision's tolerance of the exact one, so within twice
+    that of each other)."""
+    dims, mass = (4, 6, 2, 8), 0.3
+    monkeypatch.setenv("STG_MRHS_SHAPE", "14")
+    chis = torch.from_numpy(gen.source(dims, seed=3, nrhs=n)).cuda()
+    with stg.Gauge(dims, gen.gauge_field(dims, "haar", seed=1), sloppy=prec, recon=12) as g:
+        buf = torch.cat([g.pack(c, prec) for c in chis])
+        out = torch.full_like(buf, 255)
+        stg.stg_apply_A_mrhs(g.handle, n, [mass + k for k in range(n)], buf, out, prec)
+        size = out.numel() // n
+        for k in range(n):
+            got = g.unpack(out[k * size:(k + 1) * size], prec)
+            want = g.unpack(g.apply_A(g.pack(chis[k], prec), mass + k, prec), prec)
+            assert torch.linalg.vector_norm(got - want) <= 2 * tol * torch.linalg.vector_norm(want)
