@@ -277,8 +277,8 @@ stg_status stg_apply_A_dot_noalloc(const stg_gauge *g, double mass, const void *
  * per register block of NB systems, so the link traffic per system falls by
  * NB; NB (1, 2, 4, 8) and the thread-block size (128, 256) come from an
  * autotuner that times the candidates on the first call for a (lattice,
- * precision, reconstruction, nrhs) and caches the choice for the process
- * (and, when the environment variable STG_TUNE_CACHE names a file, in that
+ * precision, reconstruction, nrhs) -- of a half-pass for stg_dslash_mrhs, of A
+ * for the others -- and caches the choice for the process (and, when the environment variable STG_TUNE_CACHE names a file, in that
  * file).  prec must be FP32 or FX16 and held by the handle.
  *
  * stg_dslash_mrhs: out_k = D_{p <- 1-p} in_k for k < nrhs (Eq. 5).

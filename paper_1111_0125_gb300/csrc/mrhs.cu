@@ -34,18 +34,22 @@ void launch_dslash_m_fx16_18(int shape, int epi, const MrhsArgs &a, cudaStream_t
 // autotuner cache: process-wide, optionally mirrored in a text file named by
 // the STG_TUNE_CACHE environment variable ("Lx Ly Lz Lt prec recon n shape")
 // ---------------------------------------------------------------------------
+// what a choice was timed for: one half-pass, both half-passes of A, or either
+// (read from the file)
+enum TuneFor { TUNE_DSLASH = 0, TUNE_A = 1, TUNE_ANY = 2 };
+
 struct TuneEntry {
     int dims[4];
-    int prec, recon, nrhs, shape;
+    int prec, recon, nrhs, shape, what;
 };
 
 static std::mutex g_tune_mutex;
 static std::vector<TuneEntry> g_tune;
 static bool g_tune_loaded = false;
 
-static bool same_key(const TuneEntry &e, const int *dims, int prec, int recon, int nrhs)
+static bool same_key(const TuneEntry &e, const int *dims, int prec, int recon, int nrhs, int what)
 {
-    return e.dims[0] == dims[0] && e.dims[1] == dims[1] && e.dims[2] == dims[2] &&
+    return (e.what == TUNE_ANY || e.what == what) && e.dims[0] == dims[0] && e.dims[1] == dims[1] && e.dims[2] == dims[2] &&
            e.dims[3] == dims[3] && e.prec == prec && e.recon == recon && e.nrhs == nrhs;
 }
 
@@ -85,27 +89,28 @@ static void tune_load_file_locked()
     TuneEntry e;
     while (fscanf(f, "%d %d %d %d %d %d %d %d", &e.dims[0], &e.dims[1], &e.dims[2], &e.dims[3],
                   &e.prec, &e.recon, &e.nrhs, &e.shape) == 8) {
+        e.what = TUNE_ANY;
         if (valid_choice(e.shape)) g_tune.push_back(e);
     }
     fclose(f);
 }
 
-static bool tune_lookup(const int *dims, int prec, int recon, int nrhs, int *shape)
+static bool tune_lookup(const int *dims, int prec, int recon, int nrhs, int what, int *shape)
 {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     tune_load_file_locked();
     for (const TuneEntry &e : g_tune)
-        if (same_key(e, dims, prec, recon, nrhs)) {
+        if (same_key(e, dims, prec, recon, nrhs, what)) {
             *shape = e.shape;
             return true;
         }
     return false;
 }
 
-static void tune_store(const int *dims, int prec, int recon, int nrhs, int shape)
+static void tune_store(const int *dims, int prec, int recon, int nrhs, int what, int shape)
 {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
-    TuneEntry e = {{dims[0], dims[1], dims[2], dims[3]}, prec, recon, nrhs, shape};
+    TuneEntry e = {{dims[0], dims[1], dims[2], dims[3]}, prec, recon, nrhs, shape, what};
     g_tune.push_back(e);
     const char *path = getenv("STG_TUNE_CACHE");
     if (!path || !*path) return;
@@ -175,15 +180,23 @@ static bool forced_shape(const LinkField *lf, int n, int *shape)
     return true;
 }
 
-// Time one EPI_NONE half-pass of all n systems for every register-fed (NB,
-// threads per site) shape with TPS <= n and every staged NB (one warm-up and
-// three timed launches each, CUDA events on `s`) and keep the fastest.
-// `out` (n fields) is overwritten.
-static stg_status tune(const stg_gauge *g, const LinkField *lf, int n, const void *in, void *out,
+// Time the half-pass of all n systems, and for TUNE_A the second half-pass with
+// A's epilogue as well (the register-fed kernels lose most there: four systems
+// on 24^3x48, A 135 us with the choice for a half-pass, 102 with this one), for
+// every register-fed (NB, threads per site) shape with TPS <= n and every
+// staged NB (one warm-up and three timed rounds each, CUDA events on `s`) and
+// keep the fastest.  `out` (n fields) is overwritten.
+static stg_status tune(const stg_gauge *g, const LinkField *lf, int n, int what, const void *in, void *out,
                        size_t fstride, cudaStream_t s, int *shape_out)
 {
     if (forced_shape(lf, n, shape_out)) return STG_OK;
-    if (tune_lookup(g->dims, lf->prec, lf->recon, n, shape_out) && shape_ok(lf, *shape_out))
+    if (tune_lookup(g->dims, lf->prec, lf->recon, n, what, shape_out) && shape_ok(lf, *shape_out))
+        return STG_OK;
+    // nothing can be timed on a capturing stream: take the other choice
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone &&
+        tune_lookup(g->dims, lf->prec, lf->recon, n, what == TUNE_A ? TUNE_DSLASH : TUNE_A, shape_out) &&
+        shape_ok(lf, *shape_out))
         return STG_OK;
     cudaEvent_t e0, e1;
     STG_CUDA(cudaEventCreate(&e0));
@@ -212,15 +225,19 @@ static stg_status tune(const stg_gauge *g, const LinkField *lf, int n, const voi
             if (!shape_ok(lf, k) || (nb > 2 && nb > (n + kMsGroups - 1) / kMsGroups)) continue;
         }
         MrhsArgs a = {};
-        a.parity = 1;
         a.in = static_cast<const char *>(in);
         a.out = static_cast<char *>(out);
+        a.w = a.in;
         a.fstride = fstride;
         a.nrhs = n;
-        st = launch_m(g, lf, k, EPI_NONE, a, s);
+        for (int r = 0; r < 4 && st == STG_OK; ++r) {
+            if (r == 1) cudaEventRecord(e0, s);
+            a.parity = 1;
+            st = launch_m(g, lf, k, EPI_NONE, a, s);
+            a.parity = 0;
+            if (st == STG_OK && what == TUNE_A) st = launch_m(g, lf, k, EPI_A, a, s);
+        }
         if (st != STG_OK) break;
-        cudaEventRecord(e0, s);
-        for (int r = 0; r < 3 && st == STG_OK; ++r) st = launch_m(g, lf, k, EPI_NONE, a, s);
         cudaEventRecord(e1, s);
         ce = cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -237,7 +254,7 @@ static stg_status tune(const stg_gauge *g, const LinkField *lf, int n, const voi
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != STG_OK) return st;
-    tune_store(g->dims, lf->prec, lf->recon, n, bshape);
+    tune_store(g->dims, lf->prec, lf->recon, n, what, bshape);
     *shape_out = bshape;
     return STG_OK;
 }
@@ -590,7 +607,7 @@ stg_status batch_step(stg_batch *b)
     CGState *h = m->states_host;
     if (!b->tuned) {
         // tune NB / block size on the session's own t fields (output only)
-        STG_TRY(tune(b->g, b->lf, b->n, m->d, m->t, m->fd, s, &m->shape));
+        STG_TRY(tune(b->g, b->lf, b->n, TUNE_A, m->d, m->t, m->fd, s, &m->shape));
         b->tuned = true;
     }
     cudaGraphExec_t graph;
@@ -752,7 +769,7 @@ stg_status stg_dslash_mrhs(const stg_gauge *g, int out_parity, int nrhs, const v
     cudaStream_t s = (cudaStream_t)stream;
     const size_t fb = (size_t)g->geom.Vh * field_site_bytes(prec);
     int shape;
-    STG_TRY(tune(g, lf, nrhs, in_dev, out_dev, fb, s, &shape));
+    STG_TRY(tune(g, lf, nrhs, TUNE_DSLASH, in_dev, out_dev, fb, s, &shape));
     MrhsArgs a = {};
     a.pdl = true;
     a.parity = out_parity;
@@ -791,7 +808,7 @@ stg_status stg_apply_A_mrhs(const stg_gauge *gc, int nrhs, const double *masses,
         ws->mrhs_tmp_bytes = nrhs * fb;
     }
     int shape;
-    STG_TRY(tune(g, lf, nrhs, in_dev, ws->mrhs_tmp, fb, s, &shape));
+    STG_TRY(tune(g, lf, nrhs, TUNE_A, in_dev, ws->mrhs_tmp, fb, s, &shape));
     MrhsArgs a = {};
     a.pdl = true;
     a.parity = 1;
@@ -933,7 +950,8 @@ stg_status stg_mrhs_tuning(const stg_gauge *g, stg_prec prec, int nrhs, int *rhs
         return STG_ERR_INVALID_ARG;
     }
     int shape;
-    if (!forced_shape(lf, nrhs, &shape) && !tune_lookup(g->dims, lf->prec, lf->recon, nrhs, &shape)) {
+    if (!forced_shape(lf, nrhs, &shape) && !tune_lookup(g->dims, lf->prec, lf->recon, nrhs, TUNE_A, &shape) &&
+        !tune_lookup(g->dims, lf->prec, lf->recon, nrhs, TUNE_DSLASH, &shape)) {
         set_error("stg_mrhs_tuning: not tuned yet for this lattice, precision and nrhs");
         return STG_ERR_INVALID_ARG;
     }
