@@ -30,7 +30,44 @@ namespace stg {
 // 24^3x48, A with its dot, 18-real / 12-real: 145 / 208 us; three blocks (80
 // registers, 150-550 bytes spilled) 146 / 224 us; one block (200 registers)
 // 193 / 270 us.
-constexpr int min_blocks(int p, int r, int bs) { return (p == P64 && (r & kFixLinks) ? 2 : 1) * (kBlock / bs); }
+//
+// Other precisions have two forms with the same arithmetic: one with the
+// registers that the compiler wants (118 / 204-218 for FP32/12 and /18, 72 to 96
+// for 16 bits: two, one and three blocks per SM, the most loads in flight per
+// thread), and a dense one (80 / 128 and 64: three, two and four blocks per SM,
+// more loads in flight per SM and larger rounds of blocks).
+constexpr int min_blocks(int p, int r, int bs, bool dense)
+{
+    const int blocks = p == P64 ? (r & kFixLinks ? 2 : 1) : dense ? (p != P32 ? 4 : r == 18 ? 2 : 3) : 1;
+    return blocks * (kBlock / bs);
+}
+
+// Which form a lattice of `b` blocks of 256 sites takes: a lattice that fits
+// one round of the first form is faster there, a larger one where its rounds
+// over the 152 SMs are fewer, and FP32, FP16 and BF16 with 18-real links are
+// faster in the dense form on nearly all of those.  Measured, A with its dot, us,
+// first / dense form:
+//   blocks    256         320         375         437         525         756         864         1080        1296        1792
+//   FP32/18   14.9 / 13.6 21.4 / 16.6 25.2 / 20.0 28.3 / 23.6 35.0 / 28.3 43.9 / 37.8 48.4 / 42.2 59.0 / 51.4 70.7 / 61.3 91.4 / 81.7
+//   FP32/12    9.8 / 13.6 14.2 / 14.4 16.4 / 15.0 18.4 / 16.1 21.3 / 22.7 30.9 / 28.8 33.0 / 31.2 40.4 / 39.4 48.1 / 44.7 61.0 / 60.0
+//   FP16/18    9.4 /  9.6 13.3 / 14.9 14.4 / 15.2 16.4 / 15.5 17.5 / 15.3 26.4 / 24.0 28.3 / 26.4 33.8 / 29.8 40.6 / 36.3 51.5 / 46.1
+//   BF16/18    9.6 /  9.9 13.9 / 15.6 14.9 / 15.7 16.7 / 16.1 17.8 / 15.7 26.8 / 24.9 28.8 / 27.3 34.2 / 30.2 41.5 / 36.9 52.5 / 46.7
+//   FX16/18   12.3 / 10.2 13.0 / 16.0 13.2 / 15.5 13.7 / 16.3 17.5 / 16.3 25.0 / 25.9 26.7 / 28.2 35.5 / 31.0 38.2 / 38.0 50.4 / 48.0
+//   FP16/12   12.4 / 10.1 12.8 / 15.4 12.8 / 15.6 12.9 / 15.8 16.8 / 16.2 19.9 / 21.3 23.8 / 22.6 28.2 / 27.6 32.6 / 31.6 41.9 / 40.6
+//   BF16/12   12.9 / 10.2 13.3 / 16.0 13.4 / 16.2 13.6 / 16.6 17.5 / 17.0 20.8 / 22.5 24.4 / 23.6 29.1 / 29.0 33.5 / 33.1 43.1 / 42.4
+// (links in L2 up to 437 blocks).  With the links from memory the dense form of
+// FP16/12 at 256 blocks is the slower one, 13.7 against 13.3 us: not taken there.
+static bool dense_pays(int p, int r, int b)
+{
+    constexpr int sms = 152;
+    const auto fewer = [b](int dense, int first) {
+        return (b + dense * sms - 1) / (dense * sms) < (b + first * sms - 1) / (first * sms);
+    };
+    if (p == P64) return false;
+    if (p == P32) return r == 18 ? b >= 240 : b >= 350 && fewer(3, 2);
+    if (r == 18 && p != PX16) return b >= 425;
+    return r == 18 ? fewer(4, 3) : b >= 820;
+}
 
 // Threads per block.  Blocks of 128 put a small lattice on twice the SMs and
 // even out the last wave of a large one; between, blocks of 256 leave fewer
@@ -55,8 +92,8 @@ template <typename T> __device__ __forceinline__ T pick_m2(double d, float f);
 template <> __device__ __forceinline__ double pick_m2<double>(double d, float) { return d; }
 template <> __device__ __forceinline__ float pick_m2<float>(double, float f) { return f; }
 
-template <int P, int R, int EPI, int BS>
-__global__ void __launch_bounds__(BS, min_blocks(P, R, BS)) k_dslash(const DslashArgs a)
+template <int P, int R, int EPI, int BS, bool DENSE>
+__global__ void __launch_bounds__(BS, min_blocks(P, R, BS, DENSE)) k_dslash(const DslashArgs a)
 {
     typedef typename Real<P>::T T;
     constexpr int kUnroll = P == P64 && R == (12 | kFixLinks) && BS == kSmallBlock ? 2 : 4;  // see fix_site
@@ -117,8 +154,14 @@ template <int P, int R, int EPI>
 static void launch_bs(const DslashArgs &a, cudaStream_t s, bool pdl)
 {
     const int vh = a.g.Vh, grid = dslash_blocks(vh, EPI, P == P64 && R == (12 | kFixLinks));
-    if (grid == (vh + kBlock - 1) / kBlock) launch_k(k_dslash<P, R, EPI, kBlock>, grid, kBlock, 0, s, pdl, a);
-    else launch_k(k_dslash<P, R, EPI, kSmallBlock>, grid, kSmallBlock, 0, s, pdl, a);
+    const bool coarse = grid == (vh + kBlock - 1) / kBlock;
+    if (dense_pays(P, R, (vh + kBlock - 1) / kBlock)) {
+        if (coarse) launch_k(k_dslash<P, R, EPI, kBlock, P != P64>, grid, kBlock, 0, s, pdl, a);
+        else launch_k(k_dslash<P, R, EPI, kSmallBlock, P != P64>, grid, kSmallBlock, 0, s, pdl, a);
+    } else {
+        if (coarse) launch_k(k_dslash<P, R, EPI, kBlock, false>, grid, kBlock, 0, s, pdl, a);
+        else launch_k(k_dslash<P, R, EPI, kSmallBlock, false>, grid, kSmallBlock, 0, s, pdl, a);
+    }
 }
 
 template <int P, int R>

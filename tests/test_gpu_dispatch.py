@@ -1,5 +1,7 @@
 """Which kernel a half-pass runs: the 16-bit forms that take the one-site
 kernel give the bits of the group launch, which always runs it."""
+import functools
+
 import pytest
 import torch
 
@@ -20,6 +22,34 @@ def test_one_site_kernel_runs(dims, prec, recon):
             group = torch.empty_like(f)
             stg.stg_dslash_group([g.handle], [parity], [f], [group], prec)
             assert torch.equal(g.dslash(f, parity, prec), group)
+
+
+@functools.lru_cache(maxsize=1)
+def haar(dims):
+    return gen.gauge_field(dims, "haar", seed=5)
+
+
+@pytest.mark.parametrize("prec,recon", [(stg.STG_FP32, 12), (stg.STG_FP32, 18), (stg.STG_FP16, 12), (stg.STG_FP16, 18),
+                                        (stg.STG_BF16, 12), (stg.STG_BF16, 18), (stg.STG_FX16, 18)])
+# 16^3x32 is 256 blocks of 256 sites (dense: FP32/18), 20^3x28
+# 437.5 (dense: FP32, FP16/18, BF16/18), 20^3x34 531.25 (dense: those with 18 reals),
+# 24^3x32 864 (dense: all but FX16/18)
+@pytest.mark.parametrize("dims", [(16, 16, 16, 32), (20, 20, 20, 28), (20, 20, 20, 34), (24, 24, 24, 32)])
+def test_dense_form_gives_the_bits_of_the_group_launch(dims, prec, recon):
+    """The form with fewer registers runs the same arithmetic as the group
+    launch's sites, and its A and dot are those of its half-passes."""
+    with stg.Gauge(dims, haar(dims), sloppy=prec, recon=recon) as g:
+        f = g.pack(torch.from_numpy(gen.source(dims, seed=9)).cuda(), prec)
+        for parity in (0, 1):
+            group = torch.empty_like(f)
+            stg.stg_dslash_group([g.handle], [parity], [f], [group], prec)
+            assert torch.equal(g.dslash(f, parity, prec), group)
+        out, dot = torch.empty_like(f), torch.empty(1, dtype=torch.float64, device="cuda")
+        stg.stg_apply_A_dot(g.handle, 0.2, f, out, dot, prec)
+        assert torch.equal(out, g.apply_A(f, 0.2, prec))
+        x, y = g.unpack(f, prec), g.unpack(out, prec)
+        want = torch.sum(x.conj() * y).real
+        assert abs(dot[0] - want) <= 1e-6 * torch.sum(x.abs() * y.abs())
 
 
 @pytest.mark.parametrize("prec,recon", [(stg.STG_FP64, 18), (stg.STG_FP32, 12), (stg.STG_FP16, 12)])
