@@ -22,6 +22,8 @@
 //   EPI_A_DOT as EPI_A, plus Re sum w^dag out in FP64 -> *dot
 //   EPI_A_CG  as EPI_A inside CG, with block partials of Re sum w^dag out
 //   EPI_RES   out = w - m^2 v + D in = b - A x, plus |out|^2 in FP64 -> *dot
+#include <atomic>
+
 #include "dslash_site.cuh"
 
 namespace stg {
@@ -42,7 +44,7 @@ constexpr int min_blocks(int p, int r, int bs, bool dense)
     return blocks * (kBlock / bs);
 }
 
-// Which form a lattice of `b` blocks of 256 sites takes: a lattice that fits
+// Which of these a lattice of `b` blocks of 256 sites takes: a lattice that fits
 // one round of the first form is faster there, a larger one where its rounds
 // over the 152 SMs are fewer, and FP32, FP16 and BF16 with 18-real links are
 // faster in the dense form on nearly all of those.  Measured, A with its dot, us,
@@ -69,6 +71,25 @@ static bool dense_pays(int p, int r, int b)
     return r == 18 ? fewer(4, 3) : b >= 820;
 }
 
+// A third form starts the copy of its eight links to shared memory before it
+// waits for the previous kernel, so the links' latency overlaps that kernel's
+// end and no link load waits for registers.  It pays where its blocks (shared
+// memory for two per SM of FP32/12, one of FP32/18, four of 16 bits with 12
+// reals, three with 18) make one round.  Measured, us, other form / this one:
+//   blocks            128           256           304           375           437           531
+//   A      FP32/12     8.7 /  7.7   12.0 /  9.9   12.2 / 13.0   15.8 / 19.4   16.3 / 21.7
+//   A      FP32/18    10.0 /  7.5   14.7 / 16.0   15.1 / 18.7
+//   A      FP16/12     6.5 /  6.6   12.3 /  9.0   12.6 /  9.4   12.8 / 13.5   12.9 / 14.1
+//   A      FP16/18     8.1 /  7.2   10.7 / 10.0   11.2 / 10.7   16.0 / 12.7   16.2 / 14.4   17.2 / 18.9
+//   A pass BF16/18     2.3 /  2.1    4.8 /  3.9    5.2 /  4.1    7.5 /  4.4    7.2 /  6.1    7.8 /  9.2
+//   A pass FX16/18     2.4 /  2.2    5.8 /  4.1    6.0 /  4.2    6.2 /  4.5    6.7 /  6.3    8.0 /  9.5
+// FP32/12 at 272 blocks: 12.2 / 11.1, at 288: 12.0 / 12.3.
+static bool ahead_pays(int p, int r, int b)
+{
+    if (p == P32) return b <= (r == 18 ? 152 : 280);
+    return b <= (r == 18 ? 3 : 2) * 152;
+}
+
 // Threads per block.  Blocks of 128 put a small lattice on twice the SMs and
 // even out the last wave of a large one; between, blocks of 256 leave fewer
 // partials and share more neighbours in L1.  Measured (us, 256 against 128
@@ -92,26 +113,122 @@ template <typename T> __device__ __forceinline__ T pick_m2(double d, float f);
 template <> __device__ __forceinline__ double pick_m2<double>(double d, float) { return d; }
 template <> __device__ __forceinline__ float pick_m2<float>(double, float f) { return f; }
 
-template <int P, int R, int EPI, int BS, bool DENSE>
-__global__ void __launch_bounds__(BS, min_blocks(P, R, BS, DENSE)) k_dslash(const DslashArgs a)
+constexpr int kFirst = 0, kDense = 1, kAhead = 2;
+
+// The ahead form: every thread copies its site's eight links to its own slots
+// of shared memory, one link field of BS sites (the planes of LinkIO) for each
+// direction, forward then backward, and one commit group per direction.
+constexpr int ahead_bytes(int p, int r, int bs) { return 8 * link_bytes(p, r) * bs; }
+
+template <int N> __device__ __forceinline__ void cp_async(unsigned dst, const char *src)
+{
+    if constexpr (N == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" :: "r"(dst), "l"(src), "n"(N) : "memory");
+}
+
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
+
+// site s of a link field of vh sites to slot t of one of BS sites
+template <int B, int BS>
+__device__ __forceinline__ void cp_link(const char *dst, int t, const char *src, size_t vh, int s)
+{
+    constexpr int n = B / 16, rest = B % 16;
+    const unsigned d = smem_addr(dst);
+#pragma unroll
+    for (int q = 0; q < n; ++q) cp_async<16>(d + (q * BS + t) * 16, src + (q * vh + s) * 16);
+    if constexpr (rest != 0) cp_async<rest>(d + n * BS * 16 + t * rest, src + n * vh * 16 + (size_t)s * rest);
+}
+
+template <int P, int R, int BS>
+__device__ __forceinline__ void ahead_issue(const DslashArgs &a, const char *links, const Site &s, int i)
+{
+    constexpr int B = link_bytes(P, R);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        int jf, jb;
+        neighbours(a.g, s, i, mu, jf, jb);
+        cp_link<B, BS>(links + 2 * mu * B * BS, threadIdx.x, a.lf[mu], a.g.Vh, i);
+        cp_link<B, BS>(links + (2 * mu + 1) * B * BS, threadIdx.x, a.lb[mu], a.g.Vh, jb);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+}
+
+// dslash_site_fp with the links taken from the thread's slots
+template <int P, int R, int BS>
+__device__ __forceinline__ Vec3<float> ahead_site(const DslashArgs &a, const char *links, const Site &s, int i)
+{
+    constexpr int B = link_bytes(P, R);
+    Vec3<float> acc;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) acc.r[c] = acc.i[c] = 0.f;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        int jf, jb;
+        neighbours(a.g, s, i, mu, jf, jb);
+        float sf = 1.f, sb = 1.f;
+        if (R == 12) link_signs(a.g, s, mu, sf, sb);
+        const float s2f = R == 12 ? sf * LinkPost<P>::row2 : 1.f, s2b = R == 12 ? sb * LinkPost<P>::row2 : 1.f;
+        const Vec3<float> vf = FieldIO<P>::load_nc(a.in, a.g.Vh, jf), vb = FieldIO<P>::load_nc(a.in, a.g.Vh, jb);
+        if (mu == 0) cp_wait<3>();
+        else if (mu == 1) cp_wait<2>();
+        else if (mu == 2) cp_wait<1>();
+        else cp_wait<0>();
+        mul_add<R == 12>(LinkIO<P, R>::template load<true>(links + 2 * mu * B * BS, BS, threadIdx.x), vf, acc, s2f);
+        adj_mul_sub(LinkIO<P, R>::template load<true>(links + (2 * mu + 1) * B * BS, BS, threadIdx.x), vb, acc, s2b);
+    }
+    if (P == PX16) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            acc.r[c] *= LinkPost<PX16>::k;
+            acc.i[c] *= LinkPost<PX16>::k;
+        }
+    }
+    return acc;
+}
+
+template <int P, int R, int EPI, int BS, int FORM>
+__global__ void __launch_bounds__(BS, min_blocks(P, R, BS, FORM == kDense)) k_dslash(const DslashArgs a)
 {
     typedef typename Real<P>::T T;
     constexpr int kUnroll = P == P64 && R == (12 | kFixLinks) && BS == kSmallBlock ? 2 : 4;  // see fix_site
+    constexpr bool kReadsW = EPI != EPI_NONE && EPI != EPI_GATE;
+    extern __shared__ __align__(16) char links_ahead[];
+    const int i = blockIdx.x * BS + threadIdx.x;
+    const int vh = a.g.Vh;
+    Site site = {};
+    bool issued = false;
+    if constexpr (FORM == kAhead) {
+        if (i < vh) site = site_of(a.g, i, a.parity);
+        // links are constant, so their copies may overlap the previous kernel.
+        // The flag's writer may be that kernel: this read only decides whether
+        // to copy early, the check after the wait whether to go on.
+        issued = i < vh && ((EPI != EPI_A_CG && EPI != EPI_GATE) || *(volatile const int *)&a.state->flag == FLAG_RUN);
+        if (issued) ahead_issue<P, R, BS>(a, links_ahead, site, i);
+    }
     pdl_wait();
     pdl_trigger();
     if (EPI == EPI_A_CG || EPI == EPI_GATE) {
-        if (a.state->flag != FLAG_RUN) return;  // uniform over the grid
+        if (a.state->flag != FLAG_RUN) {  // uniform over the grid
+            if (FORM == kAhead) cp_wait<0>();
+            return;
+        }
         if (EPI == EPI_GATE && blockIdx.x == 0 && threadIdx.x == 0) cg_commit(a.state);
     }
-    const int i = blockIdx.x * BS + threadIdx.x;
-    const int vh = a.g.Vh;
     T dot = T(0);
     if (i < vh) {
-        const Vec3<T> acc = dslash_site<P, R, true, kUnroll>(a.g, a.lf, a.lb, a.parity, a.in, i);
+        Vec3<T> acc, w = {};
+        // the ahead form's waits keep later loads behind them
+        if (FORM == kAhead && kReadsW) w = FieldIO<P>::load_nc(a.w, vh, i);
+        if constexpr (FORM == kAhead) {
+            if (!issued) ahead_issue<P, R, BS>(a, links_ahead, site, i);
+            acc = ahead_site<P, R, BS>(a, links_ahead, site, i);
+        } else {
+            acc = dslash_site<P, R, true, kUnroll>(a.g, a.lf, a.lb, a.parity, a.in, i);
+        }
         if (EPI == EPI_NONE || EPI == EPI_GATE) {
             FieldIO<P>::store(a.out, vh, i, acc);
         } else if (EPI == EPI_RES) {
-            const Vec3<T> b = FieldIO<P>::load_nc(a.w, vh, i);
+            const Vec3<T> b = FORM == kAhead ? w : FieldIO<P>::load_nc(a.w, vh, i);
             const Vec3<T> x = FieldIO<P>::load_nc(a.v, vh, i);
             const T m2 = pick_m2<T>(a.m2, a.m2f);
             Vec3<T> o;
@@ -125,7 +242,7 @@ __global__ void __launch_bounds__(BS, min_blocks(P, R, BS, DENSE)) k_dslash(cons
             for (int c = 0; c < 3; ++c) dot += os.r[c] * os.r[c] + os.i[c] * os.i[c];
         } else {
             const T m2 = (EPI == EPI_A_CG) ? pick_m2<T>(a.state->m2, a.state->m2f) : pick_m2<T>(a.m2, a.m2f);
-            const Vec3<T> d = FieldIO<P>::load_nc(a.w, vh, i);
+            const Vec3<T> d = FORM == kAhead ? w : FieldIO<P>::load_nc(a.w, vh, i);
             Vec3<T> o;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -150,18 +267,48 @@ __global__ void __launch_bounds__(BS, min_blocks(P, R, BS, DENSE)) k_dslash(cons
     }
 }
 
+// The ahead form's shared memory is above the default limit and is granted per
+// device; false if it is refused (the other forms need none).  One carve-out
+// for all its instantiations: two that differ change the SMs' split between
+// consecutive kernels, 4 us more per A of FP16/12 on 16^4.
+template <int P, int R, int EPI, int BS>
+static bool ahead_granted()
+{
+    static std::atomic<unsigned long long> granted{0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev > 63) return false;
+    if (granted.load(std::memory_order_relaxed) >> dev & 1) return true;
+    const auto k = k_dslash<P, R, EPI, BS, kAhead>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, ahead_bytes(P, R, BS)) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    granted.fetch_or(1ull << dev, std::memory_order_relaxed);
+    return true;
+}
+
+template <int P, int R, int EPI, int BS>
+static void launch_form(const DslashArgs &a, int grid, cudaStream_t s, bool pdl)
+{
+    const int blocks = (a.g.Vh + kBlock - 1) / kBlock;
+    if constexpr (P != P64) {
+        if (ahead_pays(P, R, blocks) && ahead_granted<P, R, EPI, BS>()) {
+            launch_k(k_dslash<P, R, EPI, BS, kAhead>, grid, BS, ahead_bytes(P, R, BS), s, pdl, a);
+            return;
+        }
+    }
+    if (dense_pays(P, R, blocks)) launch_k(k_dslash<P, R, EPI, BS, P == P64 ? kFirst : kDense>, grid, BS, 0, s, pdl, a);
+    else launch_k(k_dslash<P, R, EPI, BS, kFirst>, grid, BS, 0, s, pdl, a);
+}
+
 template <int P, int R, int EPI>
 static void launch_bs(const DslashArgs &a, cudaStream_t s, bool pdl)
 {
     const int vh = a.g.Vh, grid = dslash_blocks(vh, EPI, P == P64 && R == (12 | kFixLinks));
-    const bool coarse = grid == (vh + kBlock - 1) / kBlock;
-    if (dense_pays(P, R, (vh + kBlock - 1) / kBlock)) {
-        if (coarse) launch_k(k_dslash<P, R, EPI, kBlock, P != P64>, grid, kBlock, 0, s, pdl, a);
-        else launch_k(k_dslash<P, R, EPI, kSmallBlock, P != P64>, grid, kSmallBlock, 0, s, pdl, a);
-    } else {
-        if (coarse) launch_k(k_dslash<P, R, EPI, kBlock, false>, grid, kBlock, 0, s, pdl, a);
-        else launch_k(k_dslash<P, R, EPI, kSmallBlock, false>, grid, kSmallBlock, 0, s, pdl, a);
-    }
+    if (grid == (vh + kBlock - 1) / kBlock) launch_form<P, R, EPI, kBlock>(a, grid, s, pdl);
+    else launch_form<P, R, EPI, kSmallBlock>(a, grid, s, pdl);
 }
 
 template <int P, int R>

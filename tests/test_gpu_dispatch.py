@@ -31,13 +31,16 @@ def haar(dims):
 
 @pytest.mark.parametrize("prec,recon", [(stg.STG_FP32, 12), (stg.STG_FP32, 18), (stg.STG_FP16, 12), (stg.STG_FP16, 18),
                                         (stg.STG_BF16, 12), (stg.STG_BF16, 18), (stg.STG_FX16, 18)])
-# 16^3x32 is 256 blocks of 256 sites (dense: FP32/18), 20^3x28
-# 437.5 (dense: FP32, FP16/18, BF16/18), 20^3x34 531.25 (dense: those with 18 reals),
-# 24^3x32 864 (dense: all but FX16/18)
-@pytest.mark.parametrize("dims", [(16, 16, 16, 32), (20, 20, 20, 28), (20, 20, 20, 34), (24, 24, 24, 32)])
-def test_dense_form_gives_the_bits_of_the_group_launch(dims, prec, recon):
-    """The form with fewer registers runs the same arithmetic as the group
-    launch's sites, and its A and dot are those of its half-passes."""
+# in blocks of 256 sites: a partial one; 81 of 128 sites; 256; 288; 375; 437.5; 531.25; 864.
+# Links copied ahead: FP32/18 up to 152, FP32/12 to 280, 16 bits to 304 (12 reals) and 456.
+# Dense: FP32/18 from 240; FP32/12 at 375, 437.5 and 864; FP16/18, BF16/18 from 531.25,
+# FX16/18 at 531.25; FP16/12, BF16/12 at 864
+@pytest.mark.parametrize("dims", [(2, 2, 2, 6), (12, 12, 12, 12), (16, 16, 16, 32), (16, 16, 18, 32), (20, 20, 20, 24),
+                                  (20, 20, 20, 28), (20, 20, 20, 34), (24, 24, 24, 32)])
+def test_every_form_gives_the_bits_of_the_group_launch(dims, prec, recon):
+    """The forms (first, fewer registers, links copied ahead) run the same
+    arithmetic as the group launch's sites; the A with the dot gives the bits
+    of the A without, and its dot that of the fields."""
     with stg.Gauge(dims, haar(dims), sloppy=prec, recon=recon) as g:
         f = g.pack(torch.from_numpy(gen.source(dims, seed=9)).cuda(), prec)
         for parity in (0, 1):
