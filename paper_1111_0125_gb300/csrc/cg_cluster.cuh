@@ -512,7 +512,7 @@ __device__ __forceinline__ const void *cl_map(const void *p, unsigned rank)
 
 // Hops of the thread's directions first_mu .. first_mu + NM - 1 in FP64 on
 // limb links lk (index parity * 4 + mu): nb: the neighbours; bits of sg: the
-// row-2 signs.
+// row-2 signs.  The 4 / NM lanes of a site decide together between integers and FP64.
 template <int RC, int NM>
 __device__ __forceinline__ Vec3<double> fix_part(const char *const *lk, int parity, int vh, int first_mu, const void *in,
                                                  int i, const int (&nb)[NM][2], unsigned sg)
@@ -524,10 +524,16 @@ __device__ __forceinline__ Vec3<double> fix_part(const char *const *lk, int pari
         const int mu = first_mu + m;
         const int s0 = (sg >> (2 * m)) & 1u ? -1 : 1, s1 = (sg >> (2 * m + 1)) & 1u ? -1 : 1;
         const Vec3<double> vf = FieldIO<P64>::load(in, vh, nb[m][0]), vb = FieldIO<P64>::load(in, vh, nb[m][1]);
-        fix_hop<false>(acc, fix_link<RC>(lk[parity * 4 + mu], vh, i, s0), vf);
-        fix_hop<true>(acc, fix_link<RC>(lk[(1 - parity) * 4 + mu], vh, nb[m][1], s1), vb);
+        fix_hop<false>(acc, fix_link<RC, false>(lk[parity * 4 + mu], vh, i, s0), vf);
+        fix_hop<true>(acc, fix_link<RC, true>(lk[(1 - parity) * 4 + mu], vh, nb[m][1], s1), vb);
     }
-    if (fix_ok(acc)) return fix_value(acc);
+    int e = acc.e;
+#pragma unroll
+    for (int o = 1; o < 4 / NM; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    unsigned t = acc.t >> min(e - acc.e, 31);
+#pragma unroll
+    for (int o = 1; o < 4 / NM; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (fix_ok(e, t)) return fix_value(acc);
     Vec3<double> d;
 #pragma unroll
     for (int c = 0; c < 3; ++c) d.r[c] = d.i[c] = 0.0;

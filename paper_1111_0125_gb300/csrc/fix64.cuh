@@ -6,31 +6,49 @@
 // times its memory time, so the mat-vecs run in fixed point instead, three
 // integer products for one FP64 product, 864 a site:
 //
-//   * A link entry is held as two limbs, u = h 2^-29 + l 2^-57, |h| <= 2^29,
-//     -2^27 <= l < 2^27 (k_fix_links, 8 bytes as the double it replaces).
-//     A link field takes this form only when every link is unitary to 1e-3
-//     (k_check_links); others keep doubles and the FP64 arithmetic.
-//   * A neighbour's colour vector is cut to 57 bits below 2^(E - 1022), E the
+//   * A link's numbers lie in memory as two limbs each, u = h 2^-29 + l 2^-57,
+//     with the bits that this cuts off beside them (fix_link.cuh).  A link
+//     field takes this form only when every link is unitary to 1e-3 and finds
+//     room for those bits (k_check_links); others keep doubles and the FP64
+//     arithmetic.
+//   * A neighbour's colour vector is cut to 57 bits below M = 2^(E - 1022), E the
 //     largest FP64 exponent met so far at this site (all limbs of a component
 //     carry its sign).  When a later neighbour raises E the sums move right.
 //   * hh sums h h' and mm sums h l' + l h' in 64 bits; the l l' terms, below
-//     2^-60 of the largest component, are left out.  Unit rows give |hh| <
-//     8 sqrt(6) 2^58 < 2^63; |mm| < 48 2^56 + 20 2^57 < 2^63.
-//   * The total hh + (mm >> 28), up to 62 bits, becomes a double once: the
-//     rounding errors of 48 FMAs (2^-53 each) are replaced by input cuts of
-//     2^-57 of the largest neighbour component and one rounding.
+//     2^-59 M, are left out.  Unit rows give |hh| < 8 sqrt(6) 2^58 < 2^63; |mm| < 48
+//     2^56 + 20 2^57 < 2^63.
+//   * The total hh + (mm >> 28), up to 62 bits, becomes a double once.
 //
-// Measured (GB300, half-pass): 32^3x64 18-real 492 -> 199 us (6.58 TB/s, 0.97
-// of the measured copy rate), 24^3x48 18-real 168 -> 66 us, 12-real 326 -> 101
-// us (issue-bound: rebuilding row 2 is 576 more products a site), 8^4 21 -> 11
-// us.  Error of D D chi on Gaussian fields against 64-bit sums: 3.4e-16 ->
-// 1.8e-16 (norm), 3.1e-15 -> 1.5e-15 (largest component).
+// These cuts are relative to M, the size of the site's largest neighbour
+// component: a component of the sum is off by at most 20 (neighbours), 48
+// (links), 12 (l l') and 2 (moved sums) times 2^-57 M, 5.1 2^-53 M, and one
+// rounding.  48 FMAs in FP64 err by up to 48 2^-53 S, S = sum |U_ab| |v_b| over
+// that component's own terms.  Where the links hardly mix the colours and
+// these differ in scale, S is far below M for the small ones.  So a site's sum
+// stands only where M <= 9 T, T a lower bound of S for every component: of six
+// numbers of a link's row against six of a neighbour, in any order, the sum of
+// products is at least m1 + c (m2 - m1), m1 and m2 the smallest and second
+// smallest of the neighbour and c the row's spread; T sums that over the eight
+// hops.  The error is then below 47 2^-53 S.  (A rebuilt row 2 errs by up to 5.1
+// 2^-57 an entry here, by several 2^-53 in FP64.)  Other sites are recomputed in FP64
+// on the links' own numbers, the arithmetic of dslash_site_fp bit for bit.
+// Gaussian neighbours on links exp(i eps H) fail the test at 2e-6 to 2e-5 of the
+// sites for eps 0.5 and 0.4; the recomputation takes some 25 us of its warp.
+// (Without the spreads it would be 1e-3, and without the 9 none.)
 //
 // Sites whose largest neighbour component is not finite, 2^1017 or more, or
-// below 2^-894 are recomputed in FP64 from the same data (zero vectors, as in
-// a point source's field, are skipped there).
+// below 2^-894 are recomputed too (zero vectors, as in a point source's field,
+// are skipped there).
+//
+// Measured (GB300, half-pass, FP64 pipe / this): 32^3x64 18-real 492 / 203 us
+// (6.46 TB/s, 0.95 of the measured copy rate), 24^3x48 18-real 168 / 65 us,
+// 12-real 326 / 100 us (issue-bound: rebuilding row 2 is 576 more products a
+// site), 8^4 21 / 11 us.  (Without the test and the bits beside the limbs: 199,
+// 62 and 98 us.)  Error of D D chi on Gaussian fields against 64-bit sums: 3.4e-16 ->
+// 1.8e-16 (norm), 3.1e-15 -> 1.5e-15 (largest component).
 #pragma once
 
+#include "fix_link.cuh"
 #include "stg_internal.h"
 
 namespace stg {
@@ -40,6 +58,7 @@ constexpr int kFixLinks = 256;
 
 struct FixLink {
     int h[3][3][2], l[3][3][2];  // [row][column][re, im]
+    unsigned c;                  // spread of the rows (columns, for a backward hop), in eighths
 };
 
 // v, in units of 2^-58, to limbs in units of 2^-29 and 2^-57
@@ -89,7 +108,7 @@ __device__ __forceinline__ void fix_row2(FixLink &u, int s)
     }
 }
 
-template <int RC, bool PLAIN = false>
+template <int RC, bool BACK>
 __device__ __forceinline__ FixLink fix_link(const char *blk, int stride, int i, int s2)
 {
     const uint4 *p = reinterpret_cast<const uint4 *>(blk) + i;
@@ -97,11 +116,12 @@ __device__ __forceinline__ FixLink fix_link(const char *blk, int stride, int i, 
     constexpr int n = RC == 18 ? 9 : 6;
 #pragma unroll
     for (int k = 0; k < n; ++k) {
-        const uint4 a = ld_link<PLAIN>(p + (size_t)k * stride);
-        u.h[k / 3][k % 3][0] = (int)a.x;
-        u.l[k / 3][k % 3][0] = (int)a.y;
-        u.h[k / 3][k % 3][1] = (int)a.z;
-        u.l[k / 3][k % 3][1] = (int)a.w;
+        const uint4 a = ld_stream(p + (size_t)k * stride);
+        u.h[k / 3][k % 3][0] = (int)a.x >> 1;
+        u.l[k / 3][k % 3][0] = (int)a.y >> 4;
+        u.h[k / 3][k % 3][1] = (int)a.z >> 1;
+        u.l[k / 3][k % 3][1] = (int)a.w >> 4;
+        if (k == 0) u.c = (BACK ? a.w : a.y) & 15u;
     }
     if (RC == 12) fix_row2(u, s2);
     return u;
@@ -110,15 +130,18 @@ __device__ __forceinline__ FixLink fix_link(const char *blk, int stride, int i, 
 struct FixAcc {
     long long hh[6], mm[6];  // re, im of colour 0, 1, 2
     int e;                   // FP64 exponent field of the scale
+    unsigned t;              // T, in units of 2^-24 M
 };
 
 constexpr int kFixExpMin = 128, kFixExpMax = 2040;
+constexpr unsigned kFixSpread = 9;  // the most that keeps 5.1 2^-53 M below 47 2^-53 S
 
 __device__ __forceinline__ void fix_init(FixAcc &a)
 {
 #pragma unroll
     for (int k = 0; k < 6; ++k) a.hh[k] = a.mm[k] = 0;
     a.e = kFixExpMin;
+    a.t = 0u;
 }
 
 // limbs of v below 2^(e - 1022): v = (h 2^28 + l) 2^(e - 1079), both with the
@@ -139,16 +162,25 @@ __device__ __forceinline__ void fix_cut(double v, int e, int &h, int &l)
     l = (xl ^ m) - m;
 }
 
+// the upper half of a double's size as a multiple of 2^-21 M, cut down (subnormals to 0)
+__device__ __forceinline__ unsigned fix_size(unsigned hi, int e)
+{
+    return ((hi & 0xfffffu) | 0x100000u) >> min(e - (int)(hi >> 20), 31);
+}
+
 // acc += U v (forward) or acc -= U^dag v (ADJ); v in doubles
 template <bool ADJ>
 __device__ __forceinline__ void fix_hop(FixAcc &acc, const FixLink &u, const Vec3<double> &v)
 {
-    unsigned mx = 0u;
+    unsigned mx = 0u, m1 = ~0u, m2 = ~0u;  // the largest, smallest and second smallest
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const unsigned a = (unsigned)__double2hiint(v.r[c]) & 0x7fffffffu;
         const unsigned b = (unsigned)__double2hiint(v.i[c]) & 0x7fffffffu;
-        mx = max(mx, max(a, b));
+        const unsigned lo = min(a, b), hi = max(a, b);
+        mx = max(mx, hi);
+        m2 = min(min(m2, hi), max(m1, lo));
+        m1 = min(m1, lo);
     }
     const int e = (int)(mx >> 20);
     if (e > acc.e) {
@@ -158,8 +190,11 @@ __device__ __forceinline__ void fix_hop(FixAcc &acc, const FixLink &u, const Vec
             acc.hh[k] >>= s;
             acc.mm[k] >>= s;
         }
+        acc.t >>= min(s, 31);
         acc.e = e;
     }
+    const unsigned n1 = fix_size(m1, acc.e);
+    acc.t += 8u * n1 + u.c * (fix_size(m2, acc.e) - n1);
     // ADJ: w = -v and its negated real parts; forward: v and its negated
     // imaginary parts
     int rh[3], rl[3], ih[3], il[3], nh[3], nl[3];
@@ -196,7 +231,10 @@ __device__ __forceinline__ void fix_hop(FixAcc &acc, const FixLink &u, const Vec
         }
 }
 
-__device__ __forceinline__ bool fix_ok(const FixAcc &a) { return a.e < kFixExpMax && a.e > kFixExpMin; }
+__device__ __forceinline__ bool fix_ok(int e, unsigned t)
+{
+    return e < kFixExpMax && e > kFixExpMin && t >= (1u << 24) / kFixSpread;
+}
 
 // (hh + (mm >> 28)) 2^(e - 1080), rounded to nearest (half away from zero) by
 // integer operations: the conversion instruction runs on the FP64 pipe
@@ -233,22 +271,27 @@ struct FixHop {
     float s;
 };
 
-// One hop in FP64 on the link's doubles (the recomputation): acc += U v, or
-// acc -= U^dag v for a backward hop.  Not inlined: it runs for exceptional
-// sites only, and inlined its registers made every site's path spill.
+// One hop in FP64 (the recomputation): acc += U v, or acc -= U^dag v for a
+// backward hop.  Not inlined: it runs for exceptional sites only, and inlined
+// its registers made every site's path spill.
 template <int RC, bool NC>
 __device__ __noinline__ void fix_hop_f64(const FixHop t, bool back, Vec3<double> *acc)
 {
     const Vec3<double> v = FieldIO<P64>::load<NC>(t.f, t.fstride, t.fi);
     if (v.r[0] == 0.0 && v.i[0] == 0.0 && v.r[1] == 0.0 && v.i[1] == 0.0 && v.r[2] == 0.0 && v.i[2] == 0.0) return;
     const uint4 *p = reinterpret_cast<const uint4 *>(t.link) + t.li;
+    int2 w[RC];
+    double n[RC];
+#pragma unroll
+    for (int k = 0; k < RC / 2; ++k) {
+        const uint4 a = ld_stream(p + (size_t)k * t.lstride);
+        w[2 * k] = make_int2((int)a.x, (int)a.y);
+        w[2 * k + 1] = make_int2((int)a.z, (int)a.w);
+    }
+    fix_decode<RC>(w, n);
     Mat3<double> u;
 #pragma unroll
-    for (int k = 0; k < (RC == 18 ? 9 : 6); ++k) {
-        const uint4 a = ld_stream(p + (size_t)k * t.lstride);
-        set_entry(u, k, (double)(int)a.x * 0x1p-29 + (double)(int)a.y * 0x1p-57,
-                  (double)(int)a.z * 0x1p-29 + (double)(int)a.w * 0x1p-57);
-    }
+    for (int k = 0; k < RC / 2; ++k) set_entry(u, k, n[2 * k], n[2 * k + 1]);
     if (RC == 12) reconstruct_row2(u, 1.0);
     const double s = RC == 12 ? (double)t.s : 1.0;
     Vec3<double> d = *acc;
@@ -271,16 +314,16 @@ __device__ __forceinline__ Vec3<double> fix_site(const Geom &g, int parity, int 
     for (int mu = 0; mu < 4; ++mu) {
         {
             const FixHop t = hop(s, i, mu, false);
-            const FixLink u = fix_link<RC>(t.link, t.lstride, t.li, t.s < 0.f ? -1 : 1);
+            const FixLink u = fix_link<RC, false>(t.link, t.lstride, t.li, t.s < 0.f ? -1 : 1);
             fix_hop<false>(acc, u, FieldIO<P64>::load<NC>(t.f, t.fstride, t.fi));
         }
         {
             const FixHop t = hop(s, i, mu, true);
-            const FixLink u = fix_link<RC>(t.link, t.lstride, t.li, t.s < 0.f ? -1 : 1);
+            const FixLink u = fix_link<RC, true>(t.link, t.lstride, t.li, t.s < 0.f ? -1 : 1);
             fix_hop<true>(acc, u, FieldIO<P64>::load<NC>(t.f, t.fstride, t.fi));
         }
     }
-    if (fix_ok(acc)) return fix_value(acc);
+    if (fix_ok(acc.e, acc.t)) return fix_value(acc);
     // from the index alone (the empty asm): no neighbour address stays in a
     // register for this branch
     asm volatile("" : "+r"(i));

@@ -10,6 +10,7 @@
 #include <new>
 #include <type_traits>
 
+#include "fix_link.cuh"
 #include "stg_internal.h"
 
 namespace stg {
@@ -156,16 +157,21 @@ stg_status pack_links_flip(const Geom &g, const double2 *ucan, int prec, int rec
 }
 
 // *bad = 1 unless every link U has |(U U^dag)_ij - delta_ij| <= 1e-3 (NaN
-// fails): the bound that the integer sums of fix64.cuh need
+// fails), the bound that the integer sums of fix64.cuh need, and fits the form
+// of fix_link.cuh with N numbers
+template <int N>
 __global__ void k_check_links(const double2 *__restrict__ ucan, long n, int *bad)
 {
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
+    double d[18];
     // FP32 is enough for the bound, and the FP64 pipe is slow
     float2 u[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         const double2 v = ucan[(size_t)k * 9 + q];
+        d[2 * q] = v.x;
+        d[2 * q + 1] = v.y;
         u[q] = make_float2((float)v.x, (float)v.y);
     }
     bool ok = true;
@@ -182,36 +188,63 @@ __global__ void k_check_links(const double2 *__restrict__ ucan, long n, int *bad
             }
             ok = ok && fabsf(re) <= 1e-3f && fabsf(im) <= 1e-3f;
         }
-    if (!ok) *bad = 1;
+    int2 w[N];
+    if (!ok || !fix_encode<N>(d, 0u, 0u, w)) *bad = 1;
 }
 
-// doubles to limbs in place: u = h 2^-29 + l 2^-57, -2^27 <= l < 2^27
-__global__ void k_fix_links(long n, double2 *u)
+// doubles to the form of fix_link.cuh in place, one thread per link
+template <int N>
+__global__ void k_fix_links(int vh, char *base, size_t blk_bytes)
 {
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const double2 v = u[k];
-    const long long a = __double2ll_rn(v.x * 0x1p57), b = __double2ll_rn(v.y * 0x1p57);
-    int4 w;
-    w.x = (int)((a + (1 << 27)) >> 28);
-    w.y = (int)(a - ((long long)w.x << 28));
-    w.z = (int)((b + (1 << 27)) >> 28);
-    w.w = (int)(b - ((long long)w.z << 28));
-    reinterpret_cast<int4 *>(u)[k] = w;
+    if (k >= 8L * vh) return;
+    double2 *p = reinterpret_cast<double2 *>(base + (size_t)(k / vh) * blk_bytes) + k % vh;
+    double u[N];
+#pragma unroll
+    for (int q = 0; q < N / 2; ++q) {
+        const double2 v = p[(size_t)q * vh];
+        u[2 * q] = v.x;
+        u[2 * q + 1] = v.y;
+    }
+    float a[3][3][2];
+#pragma unroll
+    for (int q = 0; q < N / 2; ++q) {
+        a[q / 3][q % 3][0] = fabsf((float)u[2 * q]);
+        a[q / 3][q % 3][1] = fabsf((float)u[2 * q + 1]);
+    }
+    if (N == 12) {  // row 2: sizes of the components of r0 x r1
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const int x = (c + 1) % 3, y = (c + 2) % 3;
+            const float xr = (float)u[2 * x], xi = (float)u[2 * x + 1], yr = (float)u[2 * y], yi = (float)u[2 * y + 1];
+            const float pr = (float)u[6 + 2 * x], pi = (float)u[7 + 2 * x], qr = (float)u[6 + 2 * y], qi = (float)u[7 + 2 * y];
+            a[2][c][0] = fabsf(xr * qr - xi * qi - yr * pr + yi * pi);
+            a[2][c][1] = fabsf(xr * qi + xi * qr - yr * pi - yi * pr);
+        }
+    }
+    unsigned row, col;
+    fix_spreads(a, row, col);
+    int2 w[N];
+    fix_encode<N>(u, row, col, w);  // fits: k_check_links
+#pragma unroll
+    for (int q = 0; q < N / 2; ++q)
+        reinterpret_cast<int4 *>(p)[(size_t)q * vh] = make_int4(w[2 * q].x, w[2 * q].y, w[2 * q + 1].x, w[2 * q + 1].y);
 }
 
-stg_status links_check(const double2 *ucan, long n, int *bad, cudaStream_t s)
+stg_status links_check(const double2 *ucan, long n, int recon, int *bad, cudaStream_t s)
 {
-    k_check_links<<<(int)((n + 255) / 256), 256, 0, s>>>(ucan, n, bad);
+    const int grid = (int)((n + 255) / 256);
+    if (recon == 18) k_check_links<18><<<grid, 256, 0, s>>>(ucan, n, bad);
+    else k_check_links<12><<<grid, 256, 0, s>>>(ucan, n, bad);
     STG_CUDA(cudaGetLastError());
     return STG_OK;
 }
 
-stg_status links_fix(LinkField *lf, cudaStream_t s)
+stg_status links_fix(const Geom &g, LinkField *lf, cudaStream_t s)
 {
-    // the eight blocks hold (re, im) pairs only; the padding between them goes along
-    const long n = (long)(8 * lf->blk_bytes / 16);
-    k_fix_links<<<(int)((n + 255) / 256), 256, 0, s>>>(n, reinterpret_cast<double2 *>(lf->base));
+    const int grid = (int)((8L * g.Vh + 255) / 256);
+    if (lf->recon == 18) k_fix_links<18><<<grid, 256, 0, s>>>(g.Vh, lf->base, lf->blk_bytes);
+    else k_fix_links<12><<<grid, 256, 0, s>>>(g.Vh, lf->base, lf->blk_bytes);
     STG_CUDA(cudaGetLastError());
     lf->fix = true;
     return STG_OK;
@@ -488,7 +521,7 @@ stg_status gauge_create(const int dims[4], const double *links_host, int sloppy,
     int bad = 1;
     if (st == STG_OK && (e = cudaMemsetAsync(bad_dev, 0, sizeof(int), s)) != cudaSuccess)
         st = cuda_fail(e, "cudaMemsetAsync");
-    if (st == STG_OK) st = links_check(ucan, (long)g->geom.Vh * 8, bad_dev, s);
+    if (st == STG_OK) st = links_check(ucan, (long)g->geom.Vh * 8, recon_hi, bad_dev, s);
     if (st == STG_OK && (e = cudaMemcpyAsync(&bad, bad_dev, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         st = cuda_fail(e, "cudaMemcpyAsync");
     if (st == STG_OK) st = pack_links(g->geom, ucan, P64, recon_hi, &g->hi, s);
@@ -502,7 +535,7 @@ stg_status gauge_create(const int dims[4], const double *links_host, int sloppy,
     e = cudaStreamSynchronize(s);
     if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
     if (st == STG_OK && !bad) {
-        st = links_fix(&g->hi, s);
+        st = links_fix(g->geom, &g->hi, s);
         e = cudaStreamSynchronize(s);
         if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
     }

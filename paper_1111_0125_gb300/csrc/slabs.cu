@@ -1153,7 +1153,7 @@ stg_status stg_slabs_create(const int dims[4], const double *links_host, int nsl
                                         cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) st = cuda_fail(e, "cudaMemcpyAsync(links)");
         const int t_flip = r == P - 1 ? lts - 1 : -1;
-        if (st == STG_OK) st = links_check(ucan, (long)vh * 8, bad_dev, s);
+        if (st == STG_OK) st = links_check(ucan, (long)vh * 8, prec == STG_FP64 ? recon : 18, bad_dev, s);
         if (st == STG_OK) {
             e = cudaMemcpyAsync(&bad, bad_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
             if (e != cudaSuccess) st = cuda_fail(e, "cudaMemcpyAsync");
@@ -1168,7 +1168,7 @@ stg_status stg_slabs_create(const int dims[4], const double *links_host, int nsl
     cudaFree(ucan);
     if (st == STG_OK && !bad) {
         for (int r = 0; r < P && st == STG_OK; ++r)
-            st = links_fix(prec != STG_FP64 ? &h->links64[r] : &h->links[r], s);
+            st = links_fix(h->g, prec != STG_FP64 ? &h->links64[r] : &h->links[r], s);
         h->fix = true;
     }
     if (st == STG_OK) st = sl_alloc((void **)&h->ghost, (size_t)P * 2 * h->ghost_bytes);

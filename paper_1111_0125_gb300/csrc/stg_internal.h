@@ -153,10 +153,10 @@ void cg_params_for(int sloppy, stg_cg_params *p);
 const LinkField *links_for(const stg_gauge *g, int prec);
 
 // FP64 links as limbs (gauge.cu): links_check raises *bad (device) where one
-// of n canonical links is not unitary; links_fix converts a packed FP64 field
-// in place
-stg_status links_check(const double2 *ucan, long n, int *bad, cudaStream_t s);
-stg_status links_fix(LinkField *lf, cudaStream_t s);
+// of n canonical links is not unitary or does not fit the form; links_fix
+// converts a packed FP64 field in place
+stg_status links_check(const double2 *ucan, long n, int recon, int *bad, cudaStream_t s);
+stg_status links_fix(const Geom &g, LinkField *lf, cudaStream_t s);
 
 // Reduction scratch: partial sums (one double per block) and the state.
 struct Workspace {

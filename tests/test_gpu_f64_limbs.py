@@ -6,7 +6,7 @@ Reference: the hop sum in extended precision (numpy longdouble, at least 64
 significand bits).  Bound per component, from the number formats, with v the
 largest component among the eight neighbours: cutting the neighbours to 57
 bits 2^-56 v per product, at most 8 sqrt(6) < 20 of them after unitarity
-(2^-51.6 v); links to 2^-58, 48 products (2^-52.4 v); the omitted low products
+(2^-51.6 v); links to 2^-57, 48 products (2^-51.4 v); the omitted low products
 48 2^-59 v (2^-53.4 v); one rounding of a value below 20 v (2^-48.7 v).  The
 sum is below 2^-48 v.
 """
