@@ -461,18 +461,19 @@ static stg_status cuda_check_launch()
 // ---------------------------------------------------------------------------
 stg_status launch_update_m(int pd, int vh, char *y, char *r, const char *d, const char *q, size_t sr,
                            size_t sd, CGState *states, const double *dq, double *rr, const int *active,
-                           const int *nactive, int nslots, cudaStream_t s)
+                           const int *nactive, int nslots, bool pdl, cudaStream_t s)
 {
     const dim3 grid(grid_vec(vh, nslots), nslots);
-    STG_DISPATCH_PD_EX(pd, k_cg_update_m, true, vh, y, r, d, q, sr, sd, states, dq, rr, active, nactive);
+    STG_DISPATCH_PD_EX(pd, k_cg_update_m, pdl, vh, y, r, d, q, sr, sd, states, dq, rr, active, nactive);
     return STG_OK;
 }
 
 stg_status launch_xpay_m(int pd, int vh, const char *r, char *d, size_t sr, size_t sd, CGState *states,
-                         const double *rr, const int *active, const int *nactive, int nslots, cudaStream_t s)
+                         const double *rr, const int *active, const int *nactive, int nslots, bool pdl,
+                         cudaStream_t s)
 {
     const dim3 grid(grid_vec(vh, nslots), nslots);
-    STG_DISPATCH_PD_EX(pd, k_xpay_m, true, vh, r, d, sr, sd, states, rr, active, nactive);
+    STG_DISPATCH_PD_EX(pd, k_xpay_m, pdl, vh, r, d, sr, sd, states, rr, active, nactive);
     return STG_OK;
 }
 

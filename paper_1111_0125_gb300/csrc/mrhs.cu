@@ -349,7 +349,7 @@ static stg_status iteration_m(const stg_gauge *g, MrhsWs *m, const LinkField *lf
     a.active = m->active + 1;
     a.states = m->states;
     a.partials = reinterpret_cast<float2 *>(m->partials);
-    a.pdl = true;
+    a.pdl = m->pdl;
     a.parity = 1;
     a.in = m->d;
     a.out = m->t;
@@ -362,9 +362,9 @@ static stg_status iteration_m(const stg_gauge *g, MrhsWs *m, const LinkField *lf
     const int vh = g->geom.Vh;
     double *rr = m->partials + (size_t)m->nrhs * kDqPartials;
     STG_TRY(launch_update_m(m->pd, vh, m->y, m->r, m->d, m->q, m->fr, m->fd, m->states, m->partials, rr,
-                            m->active + 1, m->active, m->nrhs, s));
+                            m->active + 1, m->active, m->nrhs, m->pdl, s));
     return launch_xpay_m(m->pd, vh, m->r, m->d, m->fr, m->fd, m->states, rr, m->active + 1, m->active,
-                         m->nrhs, s);
+                         m->nrhs, m->pdl, s);
 }
 
 static stg_status graph_m(const stg_gauge *g, MrhsWs *m, const LinkField *lf, int iters,
@@ -680,6 +680,7 @@ stg_status cg_solve_mrhs(stg_gauge *g, int n, const double *src, double *x, cons
     }
     if (!b) {
         STG_TRY(batch_create(g, n, p, s, &b));
+        b->m->pdl = true;
         ws->batch = b;
     }
     const int ctas = getenv("STG_MRHS_SHAPE") ? 0 : cluster_ctas(g, p->sloppy, n, true);

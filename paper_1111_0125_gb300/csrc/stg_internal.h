@@ -85,6 +85,12 @@ struct MrhsWs {
     cudaGraphExec_t graph = nullptr;
     int graph_iters = 0;
     int shape = 0;                    // autotuned (NB, threads per site) index
+    // The iteration's kernels by programmatic dependent launch: for a solve of
+    // its own (12^3x24 n = 8 19.6 -> 18.5 ms), not for sessions, which run side by
+    // side: waiting blocks keep places that other streams' kernels need.
+    // Served stream at 200 requests/s, three runs each, without / with: p99 744,
+    // 787, 804 / 979, 1124, 1026 ms (24^3x48 p50 558-604 / 828-945 ms).
+    bool pdl = false;
 };
 void mrhs_free(MrhsWs *m);
 void batch_destroy(stg_batch *b);
@@ -247,9 +253,10 @@ int num_sms();  // of the device current at the first call
 constexpr int kRrPartials = 384;
 stg_status launch_update_m(int pd, int vh, char *y, char *r, const char *d, const char *q, size_t sr,
                            size_t sd, CGState *states, const double *dq, double *rr, const int *active,
-                           const int *nactive, int nslots, cudaStream_t s);
+                           const int *nactive, int nslots, bool pdl, cudaStream_t s);
 stg_status launch_xpay_m(int pd, int vh, const char *r, char *d, size_t sr, size_t sd, CGState *states,
-                         const double *rr, const int *active, const int *nactive, int nslots, cudaStream_t s);
+                         const double *rr, const int *active, const int *nactive, int nslots, bool pdl,
+                         cudaStream_t s);
 stg_status launch_reset(int pd, int vh, void *y, void *r, void *d, const void *r64, double beta,
                         int copy_r, cudaStream_t s);
 stg_status launch_accumulate_x(int pr, int vh, void *x64, const void *y, cudaStream_t s);
