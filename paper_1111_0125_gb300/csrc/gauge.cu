@@ -525,6 +525,14 @@ stg_status gauge_create(const int dims[4], const double *links_host, int sloppy,
     if (st == STG_OK && (e = cudaMemcpyAsync(&bad, bad_dev, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         st = cuda_fail(e, "cudaMemcpyAsync");
     if (st == STG_OK) st = pack_links(g->geom, ucan, P64, recon_hi, &g->hi, s);
+    // The sloppy links are written last, so they lie in L2 as the packing kernel
+    // left them: loops of operators that start now run up to 1.5 times faster
+    // than on links read back from memory (A, us, with the conversion below
+    // behind the packing / this way: FP32/18 on 16^3x48 21.4 / 14.4, FP16/18 on
+    // 24^3x32 26.6 / 19.6, FP32/12 on 20^3x32 20.4 / 18.3).
+    e = cudaStreamSynchronize(s);  // the outcome of links_check
+    if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
+    if (st == STG_OK && !bad) st = links_fix(g->geom, &g->hi, s);
     if (st == STG_OK && sloppy != P64) st = pack_links(g->geom, ucan, sloppy, recon, &g->lo, s);
     if (st == STG_OK && (sloppy == PX16 || sloppy == P16) && recon == 12 && want_tiled()) {
         st = tile_links(g->geom, &g->lo, s);
@@ -534,11 +542,6 @@ stg_status gauge_create(const int dims[4], const double *links_host, int sloppy,
         st = mtile_links(g->geom, &g->lo, s);
     e = cudaStreamSynchronize(s);
     if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
-    if (st == STG_OK && !bad) {
-        st = links_fix(g->geom, &g->hi, s);
-        e = cudaStreamSynchronize(s);
-        if (st == STG_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
-    }
     cudaFree(ucan);
     if (st != STG_OK) {
         if (g->hi.base) cudaFree(g->hi.base);
