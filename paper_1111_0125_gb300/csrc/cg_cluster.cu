@@ -4,6 +4,8 @@
 #include <string.h>
 #include <time.h>
 
+#include <array>
+
 #include "cg_cluster.cuh"
 
 namespace stg {
@@ -31,29 +33,31 @@ int cluster_ctas(const stg_gauge *g, int pd, int nsys, bool batch)
     if (!g->hi.fix || !lf || nsys > kClMaxSystems) return 0;
     if (lf->fx_grid_cap > 0 || lf->fx_drop_fill) return 0;  // tests of the staged kernel
     static const int sizes[] = {16, 12, 10, 8, 6, 4};
-    struct Active {
-        int n[6];
-    };
-    static const Active active = [] {  // once, of the device current at the first call
-        Active a;
-        for (int z = 0; z < 6; ++z) a.n[z] = cl_active_clusters(sizes[z]);
+    const std::array<int, 6> active = per_device([] {
+        std::array<int, 6> a;
+        for (int z = 0; z < 6; ++z) a[z] = cl_active_clusters(sizes[z]);
         return a;
-    }();
-    if (active.n[0] < 1) return 0;
-    if (pd == P64) return vh <= 4096 ? 16 : 0;
-    if (!batch) return vh <= 16 * kClThreads ? 16 : 0;
+    });
+    if (active[0] < 1) return 0;
+    // none where the device does not grant the kernel what it needs
+    const auto granted = [&](int ctas) {
+        const int per = ctas ? (vh + ctas - 1) / ctas : 0;
+        return !ctas ? 0 : (pd == P64 || pd == P32 ? cl_granted_wide(pd, lf->recon, per) : cl_granted_16(pd, lf->recon, per)) ? ctas : 0;
+    };
+    if (pd == P64) return granted(vh <= 4096 ? 16 : 0);
+    if (!batch) return granted(vh <= 16 * kClThreads ? 16 : 0);
     double best = 16.0 + 2.0 * nsys + 3.9e-5 * nsys * (double)vh;  // the four kernels
     int ctas = 0;
     for (int z = 0; z < 6; ++z) {
-        if (active.n[z] < 1) continue;
-        const int waves = (nsys + active.n[z] - 1) / active.n[z];
+        if (active[z] < 1) continue;
+        const int waves = (nsys + active[z] - 1) / active[z];
         const double us = waves * cluster_us((vh + sizes[z] - 1) / sizes[z]);
         if (us < best) {
             best = us;
             ctas = sizes[z];
         }
     }
-    return ctas;
+    return granted(ctas);
 }
 
 // The solves of cg_solve and cg_solve_mrhs for small lattices; buf: the work

@@ -19,6 +19,7 @@
 #include <type_traits>
 
 #include "dslash_site.cuh"
+#include "per_device.h"
 
 namespace stg {
 
@@ -889,6 +890,28 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cg_cluster_one(const __grid_c
 constexpr int kClSmem = 224 * 1024;  // dynamic shared memory at most
 
 template <class K>
+static bool cl_grant(K *kernel, int smem)
+{
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+        return !smem || grant_smem(kernel, smem);
+    cudaGetLastError();
+    return false;
+}
+
+// Whether the current device grants the kernel for `per` sites per CTA
+// clusters of 16 and its shared memory.
+template <int PD, int R>
+static bool cl_granted(int per)
+{
+    constexpr int RH = PD == P64 ? R : 18;
+    if constexpr (PD != P64) {
+        if (per <= kClThreads / 4) return per_device([] { return cl_grant(k_cg_cluster_one<PD, R, 4>, kClSmem); });
+        if (per <= kClThreads) return per_device([] { return cl_grant(k_cg_cluster_one<PD, R, 1>, kClSmem); });
+    }
+    return per_device([] { return cl_grant(k_cg_cluster<PD, R, RH>, 0); });
+}
+
+template <class K>
 static cudaError_t cl_launch(K *kernel, const ClArgs &a, int nsys, int ctas, int smem, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
@@ -908,22 +931,16 @@ static cudaError_t cl_launch(K *kernel, const ClArgs &a, int nsys, int ctas, int
 template <int PD, int R, int TPS>
 static cudaError_t cl_launch_one(ClArgs a, int nsys, int ctas, cudaStream_t s)
 {
-    const auto kernel = k_cg_cluster_one<PD, R, TPS>;
-    static const cudaError_t once = [&] {  // per instantiation, thread-safe
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kClSmem);
-    }();
-    if (once != cudaSuccess) return once;
     const int per = (a.g.Vh + ctas - 1) / ctas;
     const size_t links = 16 * (((size_t)per * link_bytes(PD, R) + 15) & ~(size_t)15);
     const size_t fields = (PD == P32 ? 2 : 3) *
                           (((size_t)(per + 1) * field_site_bytes(PD) + 15) & ~(size_t)15);
     a.lsm = links + fields <= (size_t)kClSmem ? (int)links : 0;
     a.dper = make_fastdiv((unsigned)per);
-    return cl_launch(kernel, a, nsys, ctas, a.lsm + (int)fields, s);
+    return cl_launch(k_cg_cluster_one<PD, R, TPS>, a, nsys, ctas, a.lsm + (int)fields, s);
 }
 
-// the kernel for this lattice by the sites each CTA holds
+// the kernel for this lattice by the sites each CTA holds (cl_granted)
 template <int PD, int R>
 static cudaError_t cl_launch_pr(const ClArgs &a, int nsys, int ctas, cudaStream_t s)
 {
@@ -933,11 +950,7 @@ static cudaError_t cl_launch_pr(const ClArgs &a, int nsys, int ctas, cudaStream_
         if (per <= kClThreads / 4) return cl_launch_one<PD, R, 4>(a, nsys, ctas, s);
         if (per <= kClThreads) return cl_launch_one<PD, R, 1>(a, nsys, ctas, s);
     }
-    const auto kernel = k_cg_cluster<PD, R, RH>;
-    static const cudaError_t once =
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (once != cudaSuccess) return once;
-    return cl_launch(kernel, a, nsys, ctas, 0, s);
+    return cl_launch(k_cg_cluster<PD, R, RH>, a, nsys, ctas, 0, s);
 }
 
 // clusters of `ctas` CTAs that run at a time (every kernel here fills an SM's
@@ -946,7 +959,7 @@ template <int PD, int R>
 static int cl_active(int ctas)
 {
     const auto kernel = k_cg_cluster<PD, R, 18>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
+    if (!cl_grant(kernel, 0)) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctas);
     cfg.blockDim = dim3(kClThreads);
@@ -964,7 +977,9 @@ static int cl_active(int ctas)
     return n;
 }
 
-int cl_active_clusters(int ctas);
+int cl_active_clusters(int ctas);  // on the current device
+bool cl_granted_wide(int pd, int recon, int per);  // FP64, FP32
+bool cl_granted_16(int pd, int recon, int per);
 cudaError_t cl_dispatch_wide(int pd, int recon, const ClArgs &a, int nsys, int ctas, cudaStream_t s);  // FP64, FP32
 cudaError_t cl_dispatch_16(int pd, int recon, const ClArgs &a, int nsys, int ctas, cudaStream_t s);
 

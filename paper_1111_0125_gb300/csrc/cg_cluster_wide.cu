@@ -5,6 +5,12 @@ namespace stg {
 
 int cl_active_clusters(int ctas) { return cl_active<P32, 12>(ctas); }
 
+bool cl_granted_wide(int pd, int recon, int per)
+{
+    if (pd == P64) return recon == 12 ? cl_granted<P64, 12>(per) : cl_granted<P64, 18>(per);
+    return recon == 12 ? cl_granted<P32, 12>(per) : cl_granted<P32, 18>(per);
+}
+
 cudaError_t cl_dispatch_wide(int pd, int recon, const ClArgs &a, int nsys, int ctas, cudaStream_t s)
 {
     if (pd == P64)
