@@ -74,11 +74,10 @@ stg_status cluster_solve(stg_gauge *g, Workspace *ws, int ctas, int nsys, bool b
     const Geom &geo = g->geom;
     const int vh = geo.Vh;
     const bool plain = pd == P64;
-    if (!ws->cl_dev) {
-        cudaError_t e = cudaMalloc((void **)&ws->cl_dev, kClMaxSystems * sizeof(ClSystem));
-        if (e == cudaSuccess) e = cudaMallocHost((void **)&ws->cl_host, kClMaxSystems * sizeof(ClSystem));
-        if (e != cudaSuccess) return cuda_fail(e, "cluster workspace");
-    }
+    cudaError_t e = cudaSuccess;
+    if (!ws->cl_dev) e = cudaMalloc(&ws->cl_dev, kClMaxSystems * sizeof(ClSystem));
+    if (e == cudaSuccess && !ws->cl_host) e = cudaMallocHost(&ws->cl_host, kClMaxSystems * sizeof(ClSystem));
+    if (e != cudaSuccess) return cuda_fail(e, "cluster workspace");
     ClSystem *h = static_cast<ClSystem *>(ws->cl_host);
     memset(h, 0, nsys * sizeof(ClSystem));
     for (int k = 0; k < nsys; ++k) {

@@ -1,6 +1,6 @@
 """The host side of the small-lattice solves (csrc/cg_cluster.cu) against a fake
-CUDA runtime: two devices that allow different things, grants that are
-refused.  No GPU.
+CUDA runtime: two devices that allow different things, grants and allocations
+that are refused.  No GPU.
 
 The host program links the compiled cg_cluster.cu with stand-ins for the
 kernels' launchers and for the runtime calls it makes; it prints one line per
@@ -23,12 +23,13 @@ PROGRAM = r"""
 #include "cg_cluster.cuh"
 using namespace stg;
 
-static int device = 0, queries = 0;
+static int device = 0, queries = 0, fail_host = 0, launches = 0;
 // device 0: seven clusters of 16 CTAs; device 1: none; device 2: seven, kernels not granted
 extern "C" cudaError_t __wrap_cudaGetDevice(int *d) { *d = device; return cudaSuccess; }
 extern "C" cudaError_t __wrap_cudaMalloc(void **p, size_t n) { *p = calloc(1, n); return cudaSuccess; }
 extern "C" cudaError_t __wrap_cudaMallocHost(void **p, size_t n)
 {
+    if (fail_host) return cudaErrorMemoryAllocation;
     *p = calloc(1, n);
     return cudaSuccess;
 }
@@ -45,6 +46,7 @@ bool cl_granted_wide(int, int, int) { return device != 2; }
 bool cl_granted_16(int, int, int) { return device != 2; }
 cudaError_t cl_dispatch_wide(int, int, const ClArgs &a, int n, int, cudaStream_t)
 {
+    ++launches;
     for (int k = 0; k < n; ++k) a.sys[k].status = CL_OK;
     return cudaSuccess;
 }
@@ -83,6 +85,18 @@ int main(void)
     device = 0;
     check(cluster_ctas(&g, P32, 1, false) == 16, "device 0 again");
 
+    // a refused pinned allocation is an error now and no null pointer later
+    Workspace ws;
+    ClFields f = {};
+    double x = 0, mass = 0.1;
+    stg_cg_params p = {};
+    fail_host = 1;
+    check(cluster_solve(&g, &ws, 16, 1, false, f, &x, &x, &mass, 1e-10, &p, P32, nullptr, 0) != STG_OK, "refused");
+    check(cluster_solve(&g, &ws, 16, 1, false, f, &x, &x, &mass, 1e-10, &p, P32, nullptr, 0) != STG_OK,
+          "refused again");
+    fail_host = 0;
+    check(cluster_solve(&g, &ws, 16, 1, false, f, &x, &x, &mass, 1e-10, &p, P32, nullptr, 0) == STG_OK && launches == 1,
+          "granted after that");
     printf("done %d\n", bad);
     return bad != 0;
 }
