@@ -32,17 +32,6 @@ int grid_for(long n)
     return (int)(g < 1 ? 1 : g);
 }
 
-int num_sms()
-{
-    static const int n = [] {
-        int dev = 0, m = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || m <= 0) m = 148;
-        return m;
-    }();
-    return n;
-}
-
 // Per-iteration vector kernels: a grid of kVecBlocksPerSM blocks per SM
 // strides over the sites kVecUnroll at a time, issuing every load of the
 // kVecUnroll sites before the first use, so each thread keeps ~300 bytes in

@@ -19,7 +19,6 @@
 #include <type_traits>
 
 #include "dslash_site.cuh"
-#include "per_device.h"
 
 namespace stg {
 

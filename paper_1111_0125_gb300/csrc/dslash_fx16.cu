@@ -406,20 +406,12 @@ __global__ void __launch_bounds__(kFxCons, kFxCtasPerSM) k_dslash_fx2_staged(con
 template <int P, int EPI>
 static void launch_staged(const DslashArgs &a, cudaStream_t s, bool pdl)
 {
-    // set once per instantiation (thread-safe static initialisation)
-    static const int sms = [] {
-        cudaFuncSetAttribute(k_dslash_fx2_staged<P, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kFxSmem);
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-        return n;
-    }();
+    per_device([] { return grant_smem(k_dslash_fx2_staged<P, EPI>, (int)kFxSmem); });
     // a.grid_cap (STG_FX16_GRID at handle creation) caps the CTA count, so
     // that each CTA walks more tiles (tests); a.drop_fill is the failure-
     // detection test's withheld fill (a CTA's wait for its second tile runs
     // out after about a second; no fault, no hang)
-    int cap = sms * kFxCtasPerSM;
+    int cap = num_sms() * kFxCtasPerSM;
     if (a.grid_cap > 0 && a.grid_cap < cap) cap = a.grid_cap;
     const int ntiles = (a.g.Vh + kFxTile - 1) / kFxTile;
     const int grid = ntiles < cap ? ntiles : cap;

@@ -121,17 +121,6 @@ static void tune_store(const int *dims, int prec, int recon, int nrhs, int what,
     fclose(f);
 }
 
-static int num_sms_m()
-{
-    static const int n = [] {
-        int dev = 0, m = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || m <= 0) m = 148;
-        return m;
-    }();
-    return n;
-}
-
 // ---------------------------------------------------------------------------
 // launches
 // ---------------------------------------------------------------------------
@@ -139,7 +128,7 @@ static stg_status launch_m(const stg_gauge *g, const LinkField *lf, int shape, i
                            cudaStream_t s)
 {
     a.g = g->geom;
-    a.grid_cap = 2 * num_sms_m();  // blocks resident at 128 registers; they stride over tiles
+    a.grid_cap = 2 * num_sms();  // blocks resident at 128 registers; they stride over tiles
     for (int mu = 0; mu < 4; ++mu) {
         a.lf[mu] = lf->blk(a.parity, mu);
         a.lb[mu] = lf->blk(1 - a.parity, mu);

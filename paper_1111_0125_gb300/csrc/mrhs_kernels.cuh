@@ -808,22 +808,18 @@ template <int P, int NB, bool RI = false>
 void launch_ms_nb(int epi, const MrhsArgs &a, cudaStream_t s)
 {
     constexpr unsigned smem = kMsStages * ms_stage_bytes<P>();
-    // set once per instantiation (thread-safe static initialisation):
-    // resident CTAs on the whole GPU
-    static const int resident = [] {
-        cudaFuncSetAttribute(k_dslash_ms<P, NB, EPI_NONE, RI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(k_dslash_ms<P, NB, EPI_A, RI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(k_dslash_ms<P, NB, EPI_GATE, RI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(k_dslash_ms<P, NB, EPI_A_CG, RI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-            sms = 148;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dslash_ms<P, NB, EPI_A_CG, RI>, kMsThreads,
-                                                          smem) != cudaSuccess || per_sm < 1)
+    // resident CTAs on the whole device
+    const int resident = per_device([] {
+        grant_smem(k_dslash_ms<P, NB, EPI_NONE, RI>, smem);
+        grant_smem(k_dslash_ms<P, NB, EPI_A, RI>, smem);
+        grant_smem(k_dslash_ms<P, NB, EPI_GATE, RI>, smem);
+        grant_smem(k_dslash_ms<P, NB, EPI_A_CG, RI>, smem);
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dslash_ms<P, NB, EPI_A_CG, RI>, kMsThreads, smem) != cudaSuccess ||
+            per_sm < 1)
             per_sm = 1;
-        return sms * per_sm;
-    }();
+        return num_sms() * per_sm;
+    });
     const int ntiles = (a.g.Vh + kMTile - 1) / kMTile;
     int cap = resident < kDqPartials ? resident : kDqPartials;
     if (a.grid_limit > 0 && a.grid_limit < cap) cap = a.grid_limit;

@@ -227,22 +227,18 @@ template <int NB>
 void launch_msp_nb(int epi, const MrhsArgs &a, cudaStream_t s)
 {
     constexpr unsigned smem = kMspStages * ms_stage_bytes<PX16>();
-    // set once per instantiation (thread-safe static initialisation):
-    // resident CTAs on the whole GPU
-    static const int resident = [] {
-        cudaFuncSetAttribute(k_dslash_msp<NB, EPI_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(k_dslash_msp<NB, EPI_A>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(k_dslash_msp<NB, EPI_GATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(k_dslash_msp<NB, EPI_A_CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-            sms = 148;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dslash_msp<NB, EPI_A_CG>, kMspThreads,
-                                                          smem) != cudaSuccess || per_sm < 1)
+    // resident CTAs on the whole device
+    const int resident = per_device([] {
+        grant_smem(k_dslash_msp<NB, EPI_NONE>, smem);
+        grant_smem(k_dslash_msp<NB, EPI_A>, smem);
+        grant_smem(k_dslash_msp<NB, EPI_GATE>, smem);
+        grant_smem(k_dslash_msp<NB, EPI_A_CG>, smem);
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dslash_msp<NB, EPI_A_CG>, kMspThreads, smem) != cudaSuccess ||
+            per_sm < 1)
             per_sm = 1;
-        return sms * per_sm;
-    }();
+        return num_sms() * per_sm;
+    });
     const int ntiles = (a.g.Vh + kMTile - 1) / kMTile;
     int cap = resident < kDqPartials ? resident : kDqPartials;
     if (a.grid_limit > 0 && a.grid_limit < cap) cap = a.grid_limit;

@@ -34,6 +34,17 @@ auto per_device(const F &make) -> decltype(make())
     return per_device(dev, make);
 }
 
+// streaming multiprocessors of the current device
+inline int num_sms()
+{
+    const int n = per_device([] {
+        int dev = 0, m = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? m : 0;
+    });
+    return n > 0 ? n : 152;
+}
+
 // true where `kernel` may use `smem` bytes of dynamic shared memory on the
 // current device
 template <class K>

@@ -7,6 +7,7 @@
 #include <utility>
 
 #include "stg.h"
+#include "per_device.h"
 #include "stg_common.cuh"
 
 namespace stg {
@@ -245,7 +246,6 @@ struct DslashArgs {
 bool launch_dslash_16(int prec, int recon, int epi, const DslashArgs &a, cudaStream_t s, bool pdl);
 
 int grid_for(long n);
-int num_sms();  // of the device current at the first call
 
 // vector-kernel helpers with explicit operands (cg.cu)
 // dq: A's block partials of d^dag q, system k's at k times their number per
