@@ -31,7 +31,6 @@
 namespace stg {
 
 static constexpr size_t kScratchBytes = (size_t)32 << 20;
-static constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
