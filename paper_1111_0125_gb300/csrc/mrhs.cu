@@ -32,10 +32,11 @@ void launch_dslash_m_fx16_18(int shape, int epi, const MrhsArgs &a, cudaStream_t
 
 // ---------------------------------------------------------------------------
 // autotuner cache: process-wide, optionally mirrored in a text file named by
-// the STG_TUNE_CACHE environment variable ("Lx Ly Lz Lt prec recon n shape")
+// the STG_TUNE_CACHE environment variable, one line a choice: "Lx Ly Lz Lt prec
+// recon n shape what"; lines without `what` (older files) serve either use that
+// has no choice of its own
 // ---------------------------------------------------------------------------
-// what a choice was timed for: one half-pass, both half-passes of A, or either
-// (read from the file)
+// what a choice was timed for: one half-pass, both half-passes of A, or unknown
 enum TuneFor { TUNE_DSLASH = 0, TUNE_A = 1, TUNE_ANY = 2 };
 
 struct TuneEntry {
@@ -49,7 +50,7 @@ static bool g_tune_loaded = false;
 
 static bool same_key(const TuneEntry &e, const int *dims, int prec, int recon, int nrhs, int what)
 {
-    return (e.what == TUNE_ANY || e.what == what) && e.dims[0] == dims[0] && e.dims[1] == dims[1] && e.dims[2] == dims[2] &&
+    return e.what == what && e.dims[0] == dims[0] && e.dims[1] == dims[1] && e.dims[2] == dims[2] &&
            e.dims[3] == dims[3] && e.prec == prec && e.recon == recon && e.nrhs == nrhs;
 }
 
@@ -86,11 +87,13 @@ static void tune_load_file_locked()
     if (!path || !*path) return;
     FILE *f = fopen(path, "r");
     if (!f) return;
-    TuneEntry e;
-    while (fscanf(f, "%d %d %d %d %d %d %d %d", &e.dims[0], &e.dims[1], &e.dims[2], &e.dims[3],
-                  &e.prec, &e.recon, &e.nrhs, &e.shape) == 8) {
-        e.what = TUNE_ANY;
-        if (valid_choice(e.shape)) g_tune.push_back(e);
+    char line[256];
+    while (fgets(line, sizeof(line), f)) {
+        TuneEntry e;
+        const int got = sscanf(line, "%d %d %d %d %d %d %d %d %d", &e.dims[0], &e.dims[1], &e.dims[2], &e.dims[3],
+                               &e.prec, &e.recon, &e.nrhs, &e.shape, &e.what);
+        if (got == 8) e.what = TUNE_ANY;
+        if (got >= 8 && valid_choice(e.shape)) g_tune.push_back(e);
     }
     fclose(f);
 }
@@ -99,11 +102,12 @@ static bool tune_lookup(const int *dims, int prec, int recon, int nrhs, int what
 {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     tune_load_file_locked();
-    for (const TuneEntry &e : g_tune)
-        if (same_key(e, dims, prec, recon, nrhs, what)) {
-            *shape = e.shape;
-            return true;
-        }
+    for (const int use : {what, (int)TUNE_ANY})
+        for (const TuneEntry &e : g_tune)
+            if (same_key(e, dims, prec, recon, nrhs, use)) {
+                *shape = e.shape;
+                return true;
+            }
     return false;
 }
 
@@ -116,8 +120,8 @@ static void tune_store(const int *dims, int prec, int recon, int nrhs, int what,
     if (!path || !*path) return;
     FILE *f = fopen(path, "a");
     if (!f) return;
-    fprintf(f, "%d %d %d %d %d %d %d %d\n", dims[0], dims[1], dims[2], dims[3], prec, recon, nrhs,
-            shape);
+    fprintf(f, "%d %d %d %d %d %d %d %d %d\n", dims[0], dims[1], dims[2], dims[3], prec, recon, nrhs, shape,
+            what);
     fclose(f);
 }
 
