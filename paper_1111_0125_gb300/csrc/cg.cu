@@ -98,7 +98,7 @@ __device__ __forceinline__ void cg_update_body(int vh, void *y, void *r, const v
         const FF pAp = sum_partials_ff<kBlock>(dq, st->n_part);
         if (threadIdx.x == 0) {
             float a;
-            sm_ok = ff_alpha(ff_of(st->cf_delta), pAp, st->m2f, a);
+            sm_ok = ff_alpha(st->cf_delta, pAp, st->m2f, a);
             sm_alpha = T(a);
         }
     }
@@ -213,20 +213,20 @@ __device__ __forceinline__ void xpay_body(int vh, const void *r, void *d, CGStat
             }
         }
     } else {
-        const FF total = sum_partials_ff<kBlock>(rr, gridDim.x);
+        const FF total = ff_norm(sum_partials_ff<kBlock>(rr, gridDim.x));
         if (threadIdx.x == 0) {
-            const FF old = ff_of(st->cf_delta), top = ff_of(st->cf_rmax2);
-            int flag = FLAG_RUN;
-            if (!isfinite(total.hi)) flag = FLAG_BREAKDOWN;
-            else if (ff_le(total, ff_of(st->f_stop))) flag = FLAG_CONVERGED;
-            else if (st->trig2f > 0.f && ff_less(total, ff_scale(top, st->trig2f))) flag = FLAG_UPDATE;
-            else if (st->c_iter + 1 >= st->iter_limit) flag = FLAG_MAXITER;
-            sm_beta = T(ff_div(total, old));
+            const F3 old = st->cf_delta;
+            int flag = f3_stop(total, st->f_stop, st->cf_trig);
+            if (flag == FLAG_RUN && st->c_iter + 1 >= st->iter_limit) flag = FLAG_MAXITER;
+            sm_beta = T(ff_div(total, FF{old.hi, old.mid}));
             sm_run = flag == FLAG_RUN;
             if (blockIdx.x == 0) {
-                st->f_delta_old = make_float2(old.hi, old.lo);
-                st->f_delta = make_float2(total.hi, total.lo);
-                if (st->track_max && ff_less(top, total)) st->f_rmax2 = make_float2(total.hi, total.lo);
+                st->f_delta_old = old;
+                st->f_delta = F3{total.hi, total.lo, 0.f};
+                if (st->track_max && f3_cmp(total, st->cf_rmax2) > 0) {
+                    st->f_rmax2 = F3{total.hi, total.lo, 0.f};
+                    st->f_trig = f3_split(st->trig2 * ((double)total.hi + (double)total.lo));
+                }
                 st->iter = st->c_iter + 1;
                 if (flag != FLAG_RUN) st->flag = flag;
             }

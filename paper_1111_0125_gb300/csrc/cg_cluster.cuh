@@ -141,7 +141,7 @@ __device__ __forceinline__ typename ClSum<PAIR>::T cl_total(typename ClSum<PAIR>
 }
 
 // The scalars of the inner iterations, kept by thread 0 of every CTA: doubles
-// for the plain FP64 iteration, FP32 pairs otherwise (see ff_div).
+// for the plain FP64 iteration, FP32 numbers otherwise (see ff_div).
 template <bool PLAIN> struct ClScalars;
 template <> struct ClScalars<true> {
     typedef double S;
@@ -180,39 +180,37 @@ template <> struct ClScalars<true> {
 template <> struct ClScalars<false> {
     typedef FF S;
     typedef float T;
-    FF delta, delta_old, rmax2, stop;
-    float trig2, m2;
-    __device__ __forceinline__ static FF split(double v)
-    {
-        const float hi = (float)v;
-        return FF{hi, (float)(v - (double)hi)};
-    }
+    F3 delta, delta_old, rmax2, stop, trig;
+    double trig2;
+    float m2;
     __device__ __forceinline__ void start(const ClSystem &c)
     {
-        delta = split(c.delta_new);
-        delta_old = split(c.delta_old);
-        rmax2 = split(c.rmax2);
-        stop = split(c.stop);
-        trig2 = (float)c.trig2;
+        delta = f3_split(c.delta_new);
+        delta_old = f3_split(c.delta_old);
+        rmax2 = f3_split(c.rmax2);
+        stop = f3_split(c.stop);
+        trig2 = c.trig2;
+        trig = f3_split(trig2 * c.rmax2);
         m2 = (float)c.m2;
     }
     __device__ __forceinline__ void save(ClSystem &c) const
     {
-        c.delta_new = ff_double(delta);
-        c.delta_old = ff_double(delta_old);
-        c.rmax2 = ff_double(rmax2);
+        c.delta_new = f3_double(delta);
+        c.delta_old = f3_double(delta_old);
+        c.rmax2 = f3_double(rmax2);
     }
     __device__ __forceinline__ bool alpha(S pAp, T &a) const { return ff_alpha(delta, pAp, m2, a); }
-    __device__ __forceinline__ int step(S total, bool track, T &beta)
+    __device__ __forceinline__ int step(S sum, bool track, T &beta)
     {
-        int f = FLAG_RUN;
-        if (!isfinite(total.hi)) f = FLAG_BREAKDOWN;
-        else if (ff_le(total, stop)) f = FLAG_CONVERGED;
-        else if (trig2 > 0.f && ff_less(total, ff_scale(rmax2, trig2))) f = FLAG_UPDATE;
-        beta = ff_div(total, delta);
+        const FF total = ff_norm(sum);
+        const int f = f3_stop(total, stop, trig);
+        beta = ff_div(total, FF{delta.hi, delta.mid});
         delta_old = delta;
-        delta = total;
-        if (track && ff_less(rmax2, total)) rmax2 = total;
+        delta = F3{total.hi, total.lo, 0.f};
+        if (track && f3_cmp(total, rmax2) > 0) {
+            rmax2 = delta;
+            trig = f3_split(trig2 * ((double)total.hi + (double)total.lo));
+        }
         return f;
     }
 };

@@ -724,6 +724,25 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned b
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A double as three FP32 numbers in falling order, each the rest rounded to
+// nearest: all 53 bits while its last is an FP32 number (the mixed CG's sums
+// are FP32 themselves).
+struct F3 {
+    float hi, mid, lo;
+};
+
+__host__ __device__ inline F3 f3_split(double v)
+{
+    F3 r;
+    r.hi = (float)v;
+    v -= (double)r.hi;
+    r.mid = (float)v;
+    r.lo = (float)(v - (double)r.mid);
+    return r;
+}
+
+__host__ __device__ inline double f3_double(F3 a) { return (double)a.hi + ((double)a.mid + (double)a.lo); }
+
 struct CGState {
     double delta_new;  // r^dag r (iterated residual of the current precision)
     double delta_old;
@@ -742,11 +761,12 @@ struct CGState {
     int track_max;     // 1: rmax2 follows the running maximum (Sec. 3.2)
     unsigned counter;  // arrival counter of the last-block reduction
     int n_part;        // block partials of d^dag q that the update adds up
-    // Mixed CG (ff = 1): the scalars as FP32 pairs (hi, lo), which its kernels
-    // use in place of the doubles above; the host converts (state_put, state_got)
+    // Mixed CG (ff = 1): the scalars in FP32 numbers, which its kernels use in
+    // place of the doubles above; the host converts (state_put, state_got).
+    // f_trig: trig2 rmax2
     int ff;
-    float m2f, trig2f;
-    float2 f_stop, f_delta, f_delta_old, f_rmax2, cf_delta, cf_rmax2;
+    float m2f;
+    F3 f_stop, f_delta, f_delta_old, f_rmax2, f_trig, cf_delta, cf_rmax2, cf_trig;
 };
 
 // The scalars of an iteration without a last-block election.  The kernel that
@@ -788,6 +808,7 @@ __device__ __forceinline__ void cg_commit(CGState *st)
     st->c_iter = st->iter;
     st->cf_delta = st->f_delta;
     st->cf_rmax2 = st->f_rmax2;
+    st->cf_trig = st->f_trig;
 }
 
 // ---------------------------------------------------------------------------
@@ -856,30 +877,45 @@ __device__ __forceinline__ FF ff_add(FF a, FF b)
 
 __device__ __forceinline__ FF ff_of(float2 a) { return FF{a.x, a.y}; }
 
-// a < b (a <= b); exact where the pairs are close
-__device__ __forceinline__ bool ff_less(FF a, FF b) { return (a.hi - b.hi) + (a.lo - b.lo) < 0.f; }
-__device__ __forceinline__ bool ff_le(FF a, FF b) { return (a.hi - b.hi) + (a.lo - b.lo) <= 0.f; }
+// hi = the sum rounded to FP32
+__host__ __device__ __forceinline__ FF ff_norm(FF a)
+{
+    const float s = a.hi + a.lo;
+    return FF{s, a.lo - (s - a.hi)};
+}
 
-// a / b in FP32 from the pairs' 48 bits: one rounding of a quotient good to
-// 2^-46.  An FP64 division takes 1650 cycles here (its dependent steps run on
-// a pipe of 2 lanes), more than the rest of an iteration's scalars.
-__device__ __forceinline__ float ff_div(FF a, FF b)
+// a normalized pair against a triple, exactly: below 0, 0 or above as a < b, a
+// == b or a > b (rounding keeps the order, so the first parts that differ decide)
+__host__ __device__ __forceinline__ int f3_cmp(FF a, F3 b)
+{
+    if (a.hi != b.hi) return a.hi < b.hi ? -1 : 1;
+    if (a.lo != b.mid) return a.lo < b.mid ? -1 : 1;
+    return b.lo > 0.f ? -1 : b.lo < 0.f ? 1 : 0;
+}
+
+// Why an iteration of the mixed CG stops, from |r|^2 after it (its limit aside)
+__host__ __device__ __forceinline__ int f3_stop(FF total, F3 stop, F3 trig)
+{
+    if (!(total.hi - total.hi == 0.f)) return FLAG_BREAKDOWN;  // infinite, NaN
+    if (f3_cmp(total, stop) <= 0) return FLAG_CONVERGED;
+    if (trig.hi > 0.f && f3_cmp(total, trig) < 0) return FLAG_UPDATE;
+    return FLAG_RUN;
+}
+
+// a / b rounded to FP32: one rounding of a quotient good to 2^-46.  An FP64
+// division takes 1650 cycles here (its dependent steps run on a pipe of 2
+// lanes), more than the rest of an iteration's scalars.
+__host__ __device__ __forceinline__ float ff_div(FF a, FF b)
 {
     const float q = a.hi / b.hi;
     const float r = fmaf(-q, b.hi, a.hi) + fmaf(-q, b.lo, a.lo);
     return q + r / b.hi;
 }
 
-__device__ __forceinline__ FF ff_scale(FF a, float s)
-{
-    const float p = a.hi * s;
-    return FF{p, fmaf(a.hi, s, -p) + a.lo * s};
-}
-
 // alpha = delta / d^dag q of the mixed CG, with the breakdown test of cg_alpha
-__device__ __forceinline__ bool ff_alpha(FF delta, FF pAp, float m2, float &alpha)
+__device__ __forceinline__ bool ff_alpha(F3 delta, FF pAp, float m2, float &alpha)
 {
-    alpha = ff_div(delta, pAp);
+    alpha = ff_div(FF{delta.hi, delta.mid}, pAp);
     return pAp.hi > 0.f && isfinite(pAp.hi) && alpha * m2 <= 16.f;
 }
 

@@ -129,29 +129,25 @@ stg_status cuda_fail(cudaError_t e, const char *what);
 
 Geom make_geom(const int dims[4]);
 
-// The state's scalars as FP32 pairs for the mixed CG's kernels (before a copy
-// to the device, inner precision pd), and back (after one from it).
-inline float2 ff_split(double v)
-{
-    const float hi = (float)v;
-    return make_float2(hi, (float)(v - (double)hi));
-}
+// The state's scalars in FP32 numbers for the mixed CG's kernels (before a copy
+// to the device, inner precision pd), and back (after one from it); all bits
+// both ways.
 inline void state_put(CGState *h, int pd)
 {
     h->ff = pd != P64;
     h->m2f = (float)h->m2;
-    h->trig2f = (float)h->trig2;
-    h->f_stop = ff_split(h->stop_r2);
-    h->f_delta = ff_split(h->delta_new);
-    h->f_delta_old = ff_split(h->delta_old);
-    h->f_rmax2 = ff_split(h->rmax2);
+    h->f_stop = f3_split(h->stop_r2);
+    h->f_delta = f3_split(h->delta_new);
+    h->f_delta_old = f3_split(h->delta_old);
+    h->f_rmax2 = f3_split(h->rmax2);
+    h->f_trig = f3_split(h->trig2 * h->rmax2);
 }
 inline void state_got(CGState *h)
 {
     if (!h->ff) return;
-    h->delta_new = (double)h->f_delta.x + (double)h->f_delta.y;
-    h->delta_old = (double)h->f_delta_old.x + (double)h->f_delta_old.y;
-    h->rmax2 = (double)h->f_rmax2.x + (double)h->f_rmax2.y;
+    h->delta_new = f3_double(h->f_delta);
+    h->delta_old = f3_double(h->f_delta_old);
+    h->rmax2 = f3_double(h->f_rmax2);
 }
 
 // stg_cg_params defaults for inner iterations in `sloppy` (api.cu)
