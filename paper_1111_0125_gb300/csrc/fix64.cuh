@@ -20,21 +20,21 @@
 //   * The total hh + (mm >> 28), up to 62 bits, becomes a double once.
 //
 // These cuts are relative to M, the size of the site's largest neighbour
-// component: a component of the sum is off by at most 20 (neighbours), 48
-// (links), 12 (l l') and 2 (moved sums) times 2^-57 M, 5.1 2^-53 M, and one
+// component: a component of the sum is off by at most 20 (neighbours), 28
+// (links), 12 (l l') and 2 (moved sums) times 2^-57 M, 3.9 2^-53 M, and one
 // rounding.  48 FMAs in FP64 err by up to 48 2^-53 S, S = sum |U_ab| |v_b| over
 // that component's own terms.  Where the links hardly mix the colours and
 // these differ in scale, S is far below M for the small ones.  So a site's sum
-// stands only where M <= 9 T, T a lower bound of S for every component: of six
+// stands only where M <= 12 T, T a lower bound of S for every component: of six
 // numbers of a link's row against six of a neighbour, in any order, the sum of
 // products is at least m1 + c (m2 - m1), m1 and m2 the smallest and second
 // smallest of the neighbour and c the row's spread; T sums that over the eight
-// hops.  The error is then below 47 2^-53 S.  (A rebuilt row 2 errs by up to 5.1
-// 2^-57 an entry here, by several 2^-53 in FP64.)  Other sites are recomputed in FP64
-// on the links' own numbers, the arithmetic of dslash_site_fp bit for bit.
-// Gaussian neighbours on links exp(i eps H) fail the test at 2e-6 to 2e-5 of the
-// sites for eps 0.5 and 0.4; the recomputation takes some 25 us of its warp.
-// (Without the spreads it would be 1e-3, and without the 9 none.)
+// hops.  The error is then below 48 2^-53 S.  (A rebuilt row 2 errs by up to 3.5
+// 2^-57 an entry here, by several 2^-53 in FP64.)  Other sites are recomputed in
+// FP64 on the links' own numbers, the arithmetic of dslash_site_fp bit for bit;
+// that takes some 25 us of their warp.  Gaussian neighbours on links exp(i eps H)
+// fail the test at below 3e-8 of the sites for eps >= 0.3, 8e-7 for 0.2.  (With 9 for
+// 12 at 3e-6 for 0.3; without the spreads at 3e-4 for any.)
 //
 // Sites whose largest neighbour component is not finite, 2^1017 or more, or
 // below 2^-894 are recomputed too (zero vectors, as in a point source's field,
@@ -134,7 +134,7 @@ struct FixAcc {
 };
 
 constexpr int kFixExpMin = 128, kFixExpMax = 2040;
-constexpr unsigned kFixSpread = 9;  // the most that keeps 5.1 2^-53 M below 47 2^-53 S
+constexpr unsigned kFixSpread = 12;  // the most that keeps 3.9 2^-53 M below 47.5 2^-53 S
 
 __device__ __forceinline__ void fix_init(FixAcc &a)
 {

@@ -1,16 +1,17 @@
 // FP64 links as the integer Dslash reads them (fix64.cuh), without loss.
 //
 // A real number u of a link, |u| < 2, takes the 8 bytes of its double as two
-// words: u cut to a multiple of 2^-57 is h 2^-29 + l 2^-57, -2^27 <= l < 2^27; h lies in
-// the upper 31 bits of the first word and l in the upper 28 of the second.  The
-// five bits left over of each number of a link together hold what the cuts
-// took off: a number whose cut value has b significant bits lacks the last
-// 53 - b of its significand (numbers of 1/32 or more lack none), one that is cut
-// to zero takes two bits if it is zero and 65 otherwise.  Random SU(3) links
-// need 2 to 4 bits on average; the 82 (18-real) or 52 (12-real) that are there
-// suffice for all but one in about 1e10 links exp(i eps H) with eps >= 0.2.  A
-// field with a link that needs more (nearly all links close to 1, say) keeps
-// its doubles.
+// words: u rounded to a multiple of 2^-57 is h 2^-29 + l 2^-57, -2^27 <= l < 2^27; h lies
+// in the upper 31 bits of the first word and l in the upper 28 of the second.
+// The five bits left over of each number of a link together hold what the
+// rounding took off: a number whose size cut to 2^-57 has b significant bits
+// lacks the last 53 - b of its significand (numbers of 1/32 or more lack none),
+// and one bit more where the rounded value is a power of two (whether it was
+// carried there); one that is cut to zero is zero in h and l and takes two
+// bits if it is zero and 65 otherwise.  Random SU(3) links need 2 to 4 bits on
+// average; the 82 (18-real) or 52 (12-real) that are there suffice for all but
+// one in about 1e10 links exp(i eps H) with eps >= 0.2.  A field with a link that
+// needs more (nearly all links close to 1, say) keeps its doubles.
 //
 // The low four bits of the second word of numbers 0 and 1 hold the link's
 // spreads, in eighths: with the six numbers of a row in order of size, the sum
@@ -97,6 +98,15 @@ __host__ __device__ inline unsigned long long fix_units(unsigned long long bits)
     return e >= 0 ? m << e : e > -53 ? m >> -e : 0ull;
 }
 
+// the same rounded to the nearest (half away from zero; not up from zero);
+// lack: the bits of the significand below
+__host__ __device__ inline unsigned long long fix_round(unsigned long long bits, int &lack)
+{
+    const unsigned long long x = fix_units(bits);
+    lack = x ? 53 - fix_width(x) : 0;
+    return lack > 0 ? x + (bits >> (lack - 1) & 1) : x;
+}
+
 // Numbers u (each below 2 in size) to words; false, and nothing written, where
 // they do not fit.  row, col: the spreads, 0 to 15.
 template <int N> __host__ __device__ inline bool fix_encode(const double *u, unsigned row, unsigned col, int2 *w)
@@ -113,7 +123,9 @@ template <int N> __host__ __device__ inline bool fix_encode(const double *u, uns
                 pool.put(b, 64);
             }
         } else {
-            const int lack = 53 - fix_width(x);
+            int lack;
+            const unsigned long long y = fix_round(b, lack);
+            if ((y & (y - 1)) == 0 && fix_width(y) <= 53) pool.put(fix_width(y) != fix_width(x), 1);
             if (lack > 0) pool.put(b & ((1ull << lack) - 1), lack);
         }
     }
@@ -121,7 +133,8 @@ template <int N> __host__ __device__ inline bool fix_encode(const double *u, uns
 #pragma unroll
     for (int r = 0; r < N; ++r) {
         const unsigned long long b = fix_bits(u[r]);
-        const long long x = b >> 63 ? -(long long)fix_units(b) : (long long)fix_units(b);
+        int lack;
+        const long long y = (long long)fix_round(b, lack), x = b >> 63 ? -y : y;
         const int h = (int)((x + (1 << 27)) >> 28), l = (int)(x - ((long long)h << 28));
         const unsigned p = pool.of(r);
         w[r].x = (int)((unsigned)h << 1 | p >> 4);
@@ -143,9 +156,15 @@ template <int N> __host__ __device__ inline void fix_decode(const int2 *w, doubl
         if (v == 0) {
             b = pool.get(1) ? pool.get(64) : pool.get(1) << 63;
         } else {
-            const unsigned long long x = v < 0 ? (unsigned long long)-v : (unsigned long long)v;
-            const int n = fix_width(x), lack = 53 - n;
-            const unsigned long long m = lack > 0 ? x << lack | pool.get(lack) : x >> -lack;
+            const unsigned long long y = v < 0 ? (unsigned long long)-v : (unsigned long long)v;
+            int n = fix_width(y);
+            if ((y & (y - 1)) == 0 && n <= 53) n -= (int)pool.get(1);
+            const int lack = 53 - n;
+            unsigned long long m = y >> (lack < 0 ? -lack : 0);
+            if (lack > 0) {
+                const unsigned long long rest = pool.get(lack);
+                m = (y - (rest >> (lack - 1))) << lack | rest;
+            }
             b = (v < 0 ? 1ull << 63 : 0ull) | (unsigned long long)(n + 965) << 52 | (m & 0xfffffffffffffull);
         }
         memcpy(&u[r], &b, sizeof(b));

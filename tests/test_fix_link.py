@@ -1,6 +1,7 @@
 """The form in which FP64 links lie in memory for the integer Dslash
 (csrc/fix_link.cuh): every number comes back bit for bit, the limbs are the
-number cut to a multiple of 2^-57, links that do not fit are refused.
+number rounded to a multiple of 2^-57 (0 below 2^-57), links that do not fit are
+refused.
 
 A host program includes the header itself (as test_fastdiv does).  Numbers:
 uniform, with random powers of two down to the subnormals, exact 0, -0 and +-1,
@@ -42,6 +43,8 @@ template <int N> static int run(void)
             if (kind == 3) x = rnd() % 3 ? (rnd() & 1 ? 0.0 : -0.0) : (rnd() & 1 ? 1.0 : -1.0);
             if (kind == 4 && r == 5) x = ldexp(x, -(int)(rnd() % 1074));
             if (kind == 5 && rnd() % 4 == 0) x = rnd() & 1 ? 1.0005 : -1.0005;
+            if (kind == 1 && rnd() % 8 == 0)  // around a power of two: carries of the rounding
+                x = ldexp(1.0 + ((int)(rnd() % 9) - 4) * ldexp(1.0, -52), -(int)(rnd() % 12));
             u[r] = x;
         }
         const unsigned row = rnd() & 15, col = rnd() & 15;
@@ -55,8 +58,9 @@ template <int N> static int run(void)
         for (int r = 0; r < N; ++r) {
             const long long x = ((long long)(w[r].x >> 1) << 28) + (w[r].y >> 4);
             const int l = w[r].y >> 4;
+            const double y = ldexp(u[r], 57);  // llround: half away from zero
             bad += fix_bits(u[r]) != fix_bits(v[r]) || l < -(1 << 27) || l >= (1 << 27) ||
-                   x != (long long)trunc(ldexp(u[r], 57));
+                   x != (fabs(y) < 1 ? 0 : llround(y));
         }
     }
     printf("N %d bad %ld", N, bad);

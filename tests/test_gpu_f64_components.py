@@ -5,10 +5,10 @@ neighbour.
 
 Reference: the hop sum in extended precision (numpy longdouble).  Bound, with
 S = sum |U_ab| |v_b| over the 48 real products of a component: 48 FMAs err by
-up to 48 2^-53 S; the integer path by up to 5.1 2^-53 M and one rounding, and
-is taken only where M <= 12 S: 62 2^-53 S in all.  A 12-real link's row 2 is
+up to 48 2^-53 S; the integer path by up to 3.9 2^-53 M and one rounding, and
+is taken only where M <= 12 S: 48 2^-53 S in all.  A 12-real link's row 2 is
 rebuilt: in FP64 each entry errs by up to 4 2^-53 of its products' sizes (G);
-in integers by up to 5.1 2^-57, which raises 81 2^-57 M to 214 2^-57 M, 161
+in integers by up to 3.5 2^-57, which raises 62 2^-57 M to 154 2^-57 M, 116
 2^-53 S.  Where the path was integer the error is below the S terms, elsewhere
 below 48 2^-53 S and the G term.
 """
@@ -91,7 +91,7 @@ def test_components_at_different_scales(kind, bits, recon):
     U = _links(kind)
     chi = gen.source(DIMS, seed=5) * 2.0 ** -np.asarray(bits[:3])
     chi = chi.real + 1j * (chi.imag * 2.0 ** -bits[3])
-    s_bound, g_bound = (62 * 2.0 ** -53, 0.0) if recon == 18 else (161 * 2.0 ** -53, 4 * 2.0 ** -53)
+    s_bound, g_bound = (48 * 2.0 ** -53, 0.0) if recon == 18 else (116 * 2.0 ** -53, 4 * 2.0 ** -53)
     with stg.Gauge(DIMS, U, sloppy=stg.STG_FP64, recon=recon) as h:
         for parity in (0, 1):
             want, s_re, s_im, g_v = _reference(DIMS, U, chi, parity, recon)
