@@ -369,8 +369,7 @@ stg_status launch_dslash(const Geom &g, int prec, int epi, const DslashLaunch &L
             if (recon == 18) launch_pr<PB16, 18>(epi, a, s, L.pdl);
             else launch_pr<PB16, 12>(epi, a, s, L.pdl);
         } else if (prec == PX16) {
-            if (recon == 18) launch_pr<PX16, 18>(epi, a, s, L.pdl);
-            else launch_pr<PX16, 12>(epi, a, s, L.pdl);
+            launch_pr<PX16, 18>(epi, a, s, L.pdl);  // 12-real: launch_dslash_16
         } else if (recon == 18) {
             launch_pr<P16, 18>(epi, a, s, L.pdl);
         } else {

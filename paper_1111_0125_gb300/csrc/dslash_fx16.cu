@@ -422,12 +422,12 @@ static void launch_pair(int epi, const DslashArgs &a, cudaStream_t s, bool pdl)
 {
     const int grid = (a.g.Vh + 2 * kBlock - 1) / (2 * kBlock);
     switch (epi) {
-    case EPI_NONE: launch_k(k_dslash_fx2< EPI_NONE>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A: launch_k(k_dslash_fx2< EPI_A>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A_DOT: launch_k(k_dslash_fx2< EPI_A_DOT>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_A_CG: launch_k(k_dslash_fx2< EPI_A_CG>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_RES: launch_k(k_dslash_fx2< EPI_RES>, grid, kBlock, 0, s, pdl, a); break;
-    case EPI_GATE: launch_k(k_dslash_fx2< EPI_GATE>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_NONE: launch_k(k_dslash_fx2<EPI_NONE>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_A: launch_k(k_dslash_fx2<EPI_A>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_A_DOT: launch_k(k_dslash_fx2<EPI_A_DOT>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_A_CG: launch_k(k_dslash_fx2<EPI_A_CG>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_RES: launch_k(k_dslash_fx2<EPI_RES>, grid, kBlock, 0, s, pdl, a); break;
+    case EPI_GATE: launch_k(k_dslash_fx2<EPI_GATE>, grid, kBlock, 0, s, pdl, a); break;
     }
 }
 
