@@ -202,7 +202,7 @@ def test_gauge_create_rejects_bad_dims():
     assert e.value.status == stg.STG_ERR_DIMS
 
 
-@pytest.mark.parametrize("grid", ["3", None])
+@pytest.mark.parametrize("grid", ["3", "1000"])  # "1000": above the tiles, the natural grid
 def test_staged_fp16_matches_one_site_kernel(monkeypatch, grid):
     """IEEE FP16 / 12-real links also go through the staged two-site kernel
     (binary16 decode and encode in place of the fixed-point ones).  Against
@@ -213,8 +213,7 @@ def test_staged_fp16_matches_one_site_kernel(monkeypatch, grid):
     dims, mass = (12, 12, 12, 24), 0.05
     U = _links(dims, "exp", seed=4, eps=0.5)
     chi = gen.source(dims, seed=9)
-    if grid is not None:
-        monkeypatch.setenv("STG_FX16_GRID", grid)
+    monkeypatch.setenv("STG_FX16_GRID", grid)  # a set cap also keeps the staged kernel on this small lattice
     monkeypatch.setenv("STG_FX16_TILED", "0")
     plain = Gauge(dims, U, sloppy=stg.STG_FP16, recon=12)
     monkeypatch.delenv("STG_FX16_TILED")
@@ -246,7 +245,7 @@ def test_staged_fp16_matches_one_site_kernel(monkeypatch, grid):
         staged.close()
 
 
-@pytest.mark.parametrize("grid", ["1", "4", "7", None])
+@pytest.mark.parametrize("grid", ["1", "4", "7", "1000"])
 def test_staged_fx16_tiles_per_cta(monkeypatch, grid):
     """The staged FX16/12 Dslash (tile-major links streamed through shared
     memory) refills its four stages tile after tile.  A capped grid makes each
@@ -257,8 +256,7 @@ def test_staged_fx16_tiles_per_cta(monkeypatch, grid):
     dims, mass = (12, 12, 12, 24), 0.05
     U = _links(dims, "exp", seed=4, eps=0.5)
     chi = gen.source(dims, seed=9)
-    if grid is not None:
-        monkeypatch.setenv("STG_FX16_GRID", grid)
+    monkeypatch.setenv("STG_FX16_GRID", grid)  # a set cap also keeps the staged kernel on this small lattice
     monkeypatch.setenv("STG_FX16_TILED", "0")
     plain = Gauge(dims, U, sloppy=stg.STG_FX16, recon=12)
     monkeypatch.delenv("STG_FX16_TILED")
