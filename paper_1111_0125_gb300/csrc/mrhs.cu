@@ -223,6 +223,7 @@ static stg_status tune(const stg_gauge *g, const LinkField *lf, int n, int what,
         a.w = a.in;
         a.fstride = fstride;
         a.nrhs = n;
+        a.pdl = true;  // as the operators launch it
         for (int r = 0; r < 4 && st == STG_OK; ++r) {
             if (r == 1) cudaEventRecord(e0, s);
             a.parity = 1;

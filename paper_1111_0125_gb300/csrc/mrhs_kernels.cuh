@@ -800,6 +800,24 @@ __global__ void __launch_bounds__(kMsThreads, STG_MS_MINBLOCKS) k_dslash_ms(cons
     }
 }
 
+// Programmatic dependent launch of a staged kernel whose `grid` CTAs walk the
+// tiles.  A launch of its own deals its CTAs out over the SMs in turn, so the ones
+// with a tile more are spread evenly; a dependent one fills the places that
+// become free first, and some SMs get several of them.  With two rounds of
+// tiles or rounds that are full (0.9) what the early start saves is more.
+// Half-pass / A, us, dependent against ordinary: FP32/12 12^3x24 (324 tiles on 304
+// CTAs) n = 8 6.4 / 13.2 against 7.2 / 15.1, 24^3x48 (17.05 rounds) n = 16 97.9 / 217.8
+// against 99.7 / 220.0; but 16^3x32 (3.4 rounds) FP32/12 n = 16 21.5 / 48.3 against
+// 19.7 / 45.6, FX16/12 25.1 / 51.3 against 22.5 / 46.8.
+// The register-fed kernels (256-site tiles) gain up to one block per SM and lose
+// as often as they gain beyond: FX16/12 n = 2 12^3x24 (81 tiles) 4.7 / 8.9 against
+// 5.2 / 9.3, 24^3x48 26.0 / 53.5 against 24.2 / 49.7.
+inline bool staged_pdl(const MrhsArgs &a, int ntiles, int grid)
+{
+    const int rounds = (ntiles + grid - 1) / grid;
+    return a.pdl && (rounds <= 2 || 10L * ntiles >= 9L * rounds * grid);
+}
+
 // staged shapes: NB = 2, 4, 8 systems per thread and pass
 constexpr int kMrhsStagedShapes = 3;
 __host__ __device__ constexpr int ms_nb(int k) { return k == 0 ? 2 : k == 1 ? 4 : 8; }
@@ -824,11 +842,12 @@ void launch_ms_nb(int epi, const MrhsArgs &a, cudaStream_t s)
     int cap = resident < kDqPartials ? resident : kDqPartials;
     if (a.grid_limit > 0 && a.grid_limit < cap) cap = a.grid_limit;
     const int grid = ntiles < cap ? ntiles : cap;
+    const bool pdl = staged_pdl(a, ntiles, grid);
     switch (epi) {
-    case EPI_NONE: launch_k(k_dslash_ms<P, NB, EPI_NONE, RI>, grid, kMsThreads, smem, s, a.pdl, a); break;
-    case EPI_A: launch_k(k_dslash_ms<P, NB, EPI_A, RI>, grid, kMsThreads, smem, s, a.pdl, a); break;
-    case EPI_GATE: launch_k(k_dslash_ms<P, NB, EPI_GATE, RI>, grid, kMsThreads, smem, s, a.pdl, a); break;
-    case EPI_A_CG: launch_k(k_dslash_ms<P, NB, EPI_A_CG, RI>, grid, kMsThreads, smem, s, a.pdl, a); break;
+    case EPI_NONE: launch_k(k_dslash_ms<P, NB, EPI_NONE, RI>, grid, kMsThreads, smem, s, pdl, a); break;
+    case EPI_A: launch_k(k_dslash_ms<P, NB, EPI_A, RI>, grid, kMsThreads, smem, s, pdl, a); break;
+    case EPI_GATE: launch_k(k_dslash_ms<P, NB, EPI_GATE, RI>, grid, kMsThreads, smem, s, pdl, a); break;
+    case EPI_A_CG: launch_k(k_dslash_ms<P, NB, EPI_A_CG, RI>, grid, kMsThreads, smem, s, pdl, a); break;
     }
 }
 
@@ -875,11 +894,12 @@ void launch_m_pr(int shape, int epi, const MrhsArgs &a, cudaStream_t s)
         constexpr int NB_ = mrhs_nb(K_), TPS_ = mrhs_tps(K_);                                           \
         const long tiles_ = ((long)a.g.Vh * TPS_ + kMrhsBlock - 1) / kMrhsBlock;                      \
         const int grid = (int)(tiles_ < a.grid_cap ? tiles_ : a.grid_cap);                             \
+        const bool pdl = a.pdl && tiles_ <= num_sms();                                                 \
         switch (epi) {                                                                                 \
-        case EPI_NONE: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_NONE>, grid, kMrhsBlock, 0, s, a.pdl, a); break;    \
-        case EPI_A: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_A>, grid, kMrhsBlock, 0, s, a.pdl, a); break;          \
-        case EPI_GATE: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_GATE>, grid, kMrhsBlock, 0, s, a.pdl, a); break;    \
-        case EPI_A_CG: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_A_CG>, grid, kMrhsBlock, 0, s, a.pdl, a); break;    \
+        case EPI_NONE: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_NONE>, grid, kMrhsBlock, 0, s, pdl, a); break;    \
+        case EPI_A: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_A>, grid, kMrhsBlock, 0, s, pdl, a); break;          \
+        case EPI_GATE: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_GATE>, grid, kMrhsBlock, 0, s, pdl, a); break;    \
+        case EPI_A_CG: launch_k(k_dslash_m<P, R, NB_, TPS_, EPI_A_CG>, grid, kMrhsBlock, 0, s, pdl, a); break;    \
         }                                                                                              \
     } while (0)
     switch (shape) {

@@ -243,11 +243,12 @@ void launch_msp_nb(int epi, const MrhsArgs &a, cudaStream_t s)
     int cap = resident < kDqPartials ? resident : kDqPartials;
     if (a.grid_limit > 0 && a.grid_limit < cap) cap = a.grid_limit;
     const int grid = ntiles < cap ? ntiles : cap;
+    const bool pdl = staged_pdl(a, ntiles, grid);
     switch (epi) {
-    case EPI_NONE: launch_k(k_dslash_msp<NB, EPI_NONE>, grid, kMspThreads, smem, s, a.pdl, a); break;
-    case EPI_A: launch_k(k_dslash_msp<NB, EPI_A>, grid, kMspThreads, smem, s, a.pdl, a); break;
-    case EPI_GATE: launch_k(k_dslash_msp<NB, EPI_GATE>, grid, kMspThreads, smem, s, a.pdl, a); break;
-    case EPI_A_CG: launch_k(k_dslash_msp<NB, EPI_A_CG>, grid, kMspThreads, smem, s, a.pdl, a); break;
+    case EPI_NONE: launch_k(k_dslash_msp<NB, EPI_NONE>, grid, kMspThreads, smem, s, pdl, a); break;
+    case EPI_A: launch_k(k_dslash_msp<NB, EPI_A>, grid, kMspThreads, smem, s, pdl, a); break;
+    case EPI_GATE: launch_k(k_dslash_msp<NB, EPI_GATE>, grid, kMspThreads, smem, s, pdl, a); break;
+    case EPI_A_CG: launch_k(k_dslash_msp<NB, EPI_A_CG>, grid, kMspThreads, smem, s, pdl, a); break;
     }
 }
 
