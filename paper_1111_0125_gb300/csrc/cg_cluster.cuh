@@ -542,7 +542,12 @@ __device__ __forceinline__ Vec3<double> fix_part(const char *const *lk, int pari
             const float s = (sg >> (2 * m + back)) & 1u ? -1.f : 1.f;
             const FixHop h = {lk[(back ? 1 - parity : parity) * 4 + first_mu + m], vh, back ? nb[m][1] : i,
                               in, vh, nb[m][back], s};
-            fix_hop_f64<RC, false>(h, back, &d);
+            const Vec3<double> v = fix_hop_f64<RC, false>(h, back);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                d.r[c] += v.r[c];
+                d.i[c] += v.i[c];
+            }
         }
     return d;
 }

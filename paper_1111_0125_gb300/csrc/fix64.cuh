@@ -31,10 +31,12 @@
 // smallest of the neighbour and c the row's spread; T sums that over the eight
 // hops.  The error is then below 48 2^-53 S.  (A rebuilt row 2 errs by up to 3.5
 // 2^-57 an entry here, by several 2^-53 in FP64.)  Other sites are recomputed in
-// FP64 on the links' own numbers, the arithmetic of dslash_site_fp bit for bit;
-// that takes some 25 us of their warp.  Gaussian neighbours on links exp(i eps H)
-// fail the test at below 3e-8 of the sites for eps >= 0.3, 8e-7 for 0.2.  (With 9 for
-// 12 at 3e-6 for 0.3; without the spreads at 3e-4 for any.)
+// FP64 on the links' own numbers: up to four of a warp by eight lanes each, a hop
+// a lane, 3 to 4 us a site; whole warps site by site, some 25 us.  Gaussian
+// neighbours on links exp(i eps H) fail the test at below 3e-8 of the sites for eps
+// >= 0.3, 8e-7 for 0.2 (with 9 for 12 at 3e-6 for 0.3), on unit links at 3e-4.
+// Half-pass on 24^3x48 with unit links, FP64 pipe / this: Gaussian 165 / 79 us (8^4
+// 20 / 13), but real numbers only, where every site is recomputed, 165 / 324 us.
 //
 // Sites whose largest neighbour component is not finite, 2^1017 or more, or
 // below 2^-894 are recomputed too (zero vectors, as in a point source's field,
@@ -134,6 +136,7 @@ struct FixAcc {
 };
 
 constexpr int kFixExpMin = 128, kFixExpMax = 2040;
+constexpr int kFixShared = 4;       // sites of a warp recomputed by eight lanes each
 constexpr unsigned kFixSpread = 12;  // the most that keeps 3.9 2^-53 M below 47.5 2^-53 S
 
 __device__ __forceinline__ void fix_init(FixAcc &a)
@@ -271,14 +274,17 @@ struct FixHop {
     float s;
 };
 
-// One hop in FP64 (the recomputation): acc += U v, or acc -= U^dag v for a
-// backward hop.  Not inlined: it runs for exceptional sites only, and inlined
-// its registers made every site's path spill.
+// One hop in FP64 (the recomputation): U v, or -U^dag v for a backward hop.
+// Not inlined: it runs for exceptional sites only, and inlined its registers
+// made every site's path spill.
 template <int RC, bool NC>
-__device__ __noinline__ void fix_hop_f64(const FixHop t, bool back, Vec3<double> *acc)
+__device__ __noinline__ Vec3<double> fix_hop_f64(const FixHop t, bool back)
 {
     const Vec3<double> v = FieldIO<P64>::load<NC>(t.f, t.fstride, t.fi);
-    if (v.r[0] == 0.0 && v.i[0] == 0.0 && v.r[1] == 0.0 && v.i[1] == 0.0 && v.r[2] == 0.0 && v.i[2] == 0.0) return;
+    Vec3<double> d;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d.r[c] = d.i[c] = 0.0;
+    if (v.r[0] == 0.0 && v.i[0] == 0.0 && v.r[1] == 0.0 && v.i[1] == 0.0 && v.r[2] == 0.0 && v.i[2] == 0.0) return d;
     const uint4 *p = reinterpret_cast<const uint4 *>(t.link) + t.li;
     int2 w[RC];
     double n[RC];
@@ -294,10 +300,9 @@ __device__ __noinline__ void fix_hop_f64(const FixHop t, bool back, Vec3<double>
     for (int k = 0; k < RC / 2; ++k) set_entry(u, k, n[2 * k], n[2 * k + 1]);
     if (RC == 12) reconstruct_row2(u, 1.0);
     const double s = RC == 12 ? (double)t.s : 1.0;
-    Vec3<double> d = *acc;
     if (back) adj_mul_sub(u, v, d, s);
     else mul_add<RC == 12>(u, v, d, s);
-    *acc = d;
+    return d;
 }
 
 // D chi at site i; hop(s, i, mu, back) gives the eight hops' operands.  U: the
@@ -323,16 +328,47 @@ __device__ __forceinline__ Vec3<double> fix_site(const Geom &g, int parity, int 
             fix_hop<true>(acc, u, FieldIO<P64>::load<NC>(t.f, t.fstride, t.fi));
         }
     }
-    if (fix_ok(acc.e, acc.t)) return fix_value(acc);
+    const bool ok = fix_ok(acc.e, acc.t);
+    Vec3<double> d = fix_value(acc);
+    const unsigned here = __activemask(), bad = __ballot_sync(here, !ok);
+    if (bad == 0u) return d;
+    // The recomputation: the hops' vectors each by itself, added in their order.
+    if (here == 0xffffffffu && __popc(bad) <= kFixShared) {
+        // few sites of a full warp: lane k takes hop k of one site after another
+        const int k = (int)threadIdx.x & 7;
+        for (unsigned m = bad; m != 0u; m &= m - 1u) {
+            const int lane = __ffs((int)m) - 1, j = __shfl_sync(0xffffffffu, i, lane);
+            const Vec3<double> h = fix_hop_f64<RC, NC>(hop(site_of(g, j, parity), j, k >> 1, k & 1), k & 1);
+            Vec3<double> sum;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sum.r[c] = sum.i[c] = 0.0;
+#pragma unroll 1
+            for (int n = 0; n < 8; ++n)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    sum.r[c] += __shfl_sync(0xffffffffu, h.r[c], n);
+                    sum.i[c] += __shfl_sync(0xffffffffu, h.i[c], n);
+                }
+            if (((int)threadIdx.x & 31) == lane) d = sum;
+        }
+        return d;
+    }
+    if (ok) return d;
     // from the index alone (the empty asm): no neighbour address stays in a
     // register for this branch
     asm volatile("" : "+r"(i));
     const Site z = site_of(g, i, parity);
-    Vec3<double> d;
 #pragma unroll
     for (int c = 0; c < 3; ++c) d.r[c] = d.i[c] = 0.0;
 #pragma unroll 1
-    for (int k = 0; k < 8; ++k) fix_hop_f64<RC, NC>(hop(z, i, k >> 1, k & 1), k & 1, &d);
+    for (int k = 0; k < 8; ++k) {
+        const Vec3<double> h = fix_hop_f64<RC, NC>(hop(z, i, k >> 1, k & 1), k & 1);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            d.r[c] += h.r[c];
+            d.i[c] += h.i[c];
+        }
+    }
     return d;
 }
 
