@@ -219,8 +219,9 @@ stg_status stg_dslash(const stg_gauge *g, int out_parity, const void *in_dev,
  * handles may hold lattices of different sizes but must share the device
  * and the reconstruction (18 or 12) of their links in `prec`.  Each item's
  * output is bitwise the one of stg_dslash where that runs the one-site-per-
- * thread kernel (every precision but FX16 / 12-real, whose stg_dslash runs
- * the packed staged kernel: agreement to rounding); the group runs as one
+ * thread kernel (every precision but FX16 / 12-real and, on large lattices,
+ * FP16 / 12-real, whose stg_dslash runs packed kernels: agreement to
+ * rounding); the group runs as one
  * grid, which fills the GPU where one small lattice would not.  Arrays
  * are host arrays of n entries; fields as for stg_dslash.  No item's output
  * may alias any item's input: an output pointer equal to any in_dev[j]
@@ -264,7 +265,7 @@ stg_status stg_apply_A_dot(const stg_gauge *g, double mass, const void *in_dev,
  *   Arguments as for stg_apply_A_dot; the handle must already exist (its
  *   links were allocated by stg_gauge_create).
  *   Limit: 48 Vh (FP64), 24 Vh (FP32) or 16 Vh (FP16, FX16, BF16) bytes plus 8
- *   bytes per 256 sites must fit in 32 MiB (FP64 up to 24^3x48, the others
+ *   bytes per 256 sites (per 128 up to 16384 sites) must fit in 32 MiB (FP64 up to 24^3x48, the others
  *   up to 32^3x64); larger lattices return STG_ERR_INVALID_ARG with a message.
  *   The first call on a device looks up the array's device address (once per
  *   device); make that first call before any stream capture.
@@ -284,8 +285,9 @@ stg_status stg_apply_A_dot_noalloc(const stg_gauge *g, double mass, const void *
  * NB; NB (1, 2, 4, 8) and the thread-block size (128, 256) come from an
  * autotuner that times the candidates on the first call for a (lattice,
  * precision, reconstruction, nrhs) -- of a half-pass for stg_dslash_mrhs, of A
- * for the others -- and caches the choice for the process (and, when the environment variable STG_TUNE_CACHE names a file, in that
- * file).  prec must be FP32 or FX16 and held by the handle.
+ * for the others -- and caches the choice for the process (and, when the
+ * environment variable STG_TUNE_CACHE names a file, in that file, with what it
+ * was timed for).  prec must be FP32 or FX16 and held by the handle.
  *
  * stg_dslash_mrhs: out_k = D_{p <- 1-p} in_k for k < nrhs (Eq. 5).
  */

@@ -29,9 +29,9 @@
 namespace stg {
 
 // Limb links (fix64.cuh): two blocks per SM, 128 registers.  Measured at
-// 24^3x48, A with its dot, 18-real / 12-real: 145 / 208 us; three blocks (80
-// registers, 150-550 bytes spilled) 146 / 224 us; one block (200 registers)
-// 193 / 270 us.
+// 24^3x48, A with its dot, 18-real / 12-real: 148 / 214 us; before the limbs carried
+// all bits of a link 145 / 208 us, against 146 / 224 us with three blocks (80
+// registers, 150-550 bytes spilled) and 193 / 270 us with one (200 registers).
 //
 // Other precisions have two forms with the same arithmetic: one with the
 // registers that the compiler wants (118 / 204-218 for FP32/12 and /18, 72 to 96

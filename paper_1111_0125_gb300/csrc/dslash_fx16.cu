@@ -453,7 +453,10 @@ static void launch_staged_p(int epi, const DslashArgs &a, cudaStream_t s, bool p
 // FP16/12, us, staged against one site per thread): Vh 20736: 6.9 / 15.8
 // against 2.7 / 7.5; 65536: 7.2 / 18.5 against 4.4 / 10.7; 331776: 18.5 / 39.7
 // against 14.5 / 33.8; 786432 (5.05 rounds): 32.0 / 67.3 against 30.1 / 67.8;
-// 1048576 (6.74): 37.3 / 79.2 against 39.2 / 87.7.  The capped and the
+// 1048576 (6.74): 37.3 / 79.2 against 39.2 / 87.7.  FX16/12, staged against the
+// packed kernel: 20736: 7.3 / 16.8 against 3.6 / 9.5; 65536: 7.3 / 17.0 against 4.4 /
+// 11.2; 331776: 19.4 / 41.7 against 15.2 / 35.6; 526848: 24.6 / 52.5 against 21.1 / 48.3;
+// 786432: 33.7 / 71.7 against 29.9 / 69.8.  The capped and the
 // withheld-fill grids of the tests always run staged.
 static bool staged_pays(const DslashArgs &a)
 {

@@ -45,7 +45,7 @@
 // Measured (GB300, half-pass, FP64 pipe / this): 32^3x64 18-real 492 / 203 us
 // (6.46 TB/s, 0.95 of the measured copy rate), 24^3x48 18-real 168 / 65 us,
 // 12-real 326 / 100 us (issue-bound: rebuilding row 2 is 576 more products a
-// site), 8^4 21 / 11 us.  (Without the test and the bits beside the limbs: 199,
+// site), 8^4 20 / 6.2 us.  (Without the test and the bits beside the limbs: 199,
 // 62 and 98 us.)  Error of D D chi on Gaussian fields against 64-bit sums: 3.4e-16 ->
 // 1.8e-16 (norm), 3.1e-15 -> 1.5e-15 (largest component).
 #pragma once
